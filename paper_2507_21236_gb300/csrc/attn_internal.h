@@ -85,6 +85,7 @@ struct attn_ctx {
   uint64_t launches = 0;
   int device = 0;
   int num_sms = 0;
+  size_t total_mem = 0;
   // Scratch areas reused across calls (grow only). Every reallocation of one of
   // them bumps scratch_epoch: a captured eigensolve graph records the epoch it was
   // built under and is rebuilt when it differs (its kernels hold the old addresses).
@@ -96,6 +97,7 @@ struct attn_ctx {
   attn::DevBuf oz_ws[4];  // split-GEMM operand slices and row exponents (P slices, P exps, Q slices, Q exps)
   attn::DevBuf oz_err;    // split-GEMM device error word
   bool oz_err_init = false;
+  size_t dense_bytes = 0; // device memory of the dense pair operators of this context's H_effs
   // Optional per-kernel timing (attn_profile_enable): event pairs around launches.
   bool prof_on = false;
   struct ProfRec {

@@ -192,6 +192,7 @@ ATTN_API attn_status attn_create(const attn_config* cfg, void* stream, attn_ctx*
   ATTN_REQUIRE(prop.major == 10 && prop.minor == 3, ATTN_ECUDA,
                std::string("libattn is built for sm_103a only; device is ") + prop.name);
   ctx->num_sms = prop.multiProcessorCount;
+  ctx->total_mem = prop.totalGlobalMem;
   // NULL selects the legacy default stream (what torch's default stream reports as 0)
   ctx->stream = stream ? (cudaStream_t)stream : (cudaStream_t)0;
   ctx->own_stream = false;
@@ -653,6 +654,7 @@ static void eigsolve_dev(attn_heff* h, double* T_dev, double* theta, int* iters)
   MatVec lo = [&](const double* a, double* b) { h->apply(a, b, dt); };
   MatVec hi = [&](const double* a, double* b) { h->apply_f64(a, b); };
   const int rsteps = (dt != ATTN_F64) ? cfg.refine_steps : 0;
+  h->expect = dt == ATTN_F64 ? cfg.lanczos_depth : 1 + std::max(rsteps, 0);
   if (cfg.use_graphs) {
     EigGraph* g = h->eg;
     // a graph holds the addresses of the context's scratch buffers at capture time:

@@ -2,6 +2,7 @@
 #pragma once
 
 #include "attn_internal.h"
+#include "heff_dense.h"
 #include "lanczos.h"
 
 // A captured CUDA graph of one eigensolve (Lanczos + optional FP64 refinement)
@@ -47,6 +48,10 @@ struct attn_heff {
   // Low-precision tensor-core copies, built at the first application in that type:
   // tc[0] BF16 operands, tc[1] TF32 operands (opaque, owned by heff_tc.cu).
   void* tc[2] = {nullptr, nullptr};
+  // FP64 operators summed per link pair, once they pay (heff_dense.cu): applications made,
+  // and how many the caller of the next ones announces (a Lanczos its depth)
+  attn::DenseF64* dense = nullptr;
+  int f64_uses = 0, expect = 1;
   EigGraph* eg = nullptr; // cached eigensolve graph (use_graphs)
   attn::DevBuf host_x;    // device copy of the tensor of attn_eigsolve_host
   double flops() const;

@@ -1,0 +1,471 @@
+// H_eff applied through one dense operator per link pair (Sec. 3.3.2: the products of a
+// node summed before they meet the tensor).
+//
+// The pair products of kind (p, q) act on the joint index of two links only, so their sum
+//     M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j']   (+ H_p[i][i'] delta_jj' + delta_ii' H_q[j][j'])
+// is one PQ x PQ matrix, and an application to a tensor with S slices costs 2 (PQ)^2 S
+// operations instead of 2 R (P + Q) PQ S: less as soon as R > PQ / (P + Q) products share the
+// pair (64 at 128 x 128; the nodes of the 8x8 to 32x32 lattices have 50 to 300). Making M
+// costs 2 R (PQ)^2, about half of one product-by-product application, once per H_eff.
+//
+// FP64 on the CUDA cores. This GPU executes two FP64 FMAs per SM and cycle, so the number of
+// FMAs decides (M streams from L2 or HBM far below their rates), and a simple kernel saturates
+// it: every CTA owns a block of y and adds the contributions of all three pair kinds to it,
+// in a fixed order, with no workspace and no second launch. Measured (GB300, one
+// application): [64]^3 with 140 products per pair 25.4 -> 5.6 ms; [16]^3 with 12
+// 128 -> 16 us, where the product-by-product path spends its time on 17 launches.
+#include <algorithm>
+
+#include "heff.h"
+#include "heff_dense.h"
+
+namespace attn {
+
+namespace {
+
+// ---------------------------------------------------------------- the operators
+struct PairOp {
+  const double* a;   // [R][P][P]
+  const double* b;   // [R][Q][Q]
+  const double* hp;  // internal operator on slot p, or null
+  const double* hq;
+  double* m;         // [P Q][P Q]
+  int P, Q, R;
+  int tiles_n, tile0;  // column tiles, first tile of this kind
+};
+struct PairOps {
+  PairOp k[3];
+  int n;
+};
+
+// M as a P^2 x Q^2 GEMM over the products (rows (i, i'), columns (j, j')); both operand
+// stacks are contiguous along the output index, so no transpose is needed. 64 x 64 tiles,
+// 4 x 4 per thread, 16 products per step.
+constexpr int kBT = 64, kBK = 16;
+__global__ void __launch_bounds__(256) pair_operator_kernel(const PairOps ops) {
+  __shared__ double As[kBK][kBT], Bs[kBK][kBT];
+  int ki = 0;
+  if (ops.n > 1 && (int)blockIdx.x >= ops.k[1].tile0) ki = 1;
+  if (ops.n > 2 && (int)blockIdx.x >= ops.k[2].tile0) ki = 2;
+  const PairOp o = ki == 0 ? ops.k[0] : (ki == 1 ? ops.k[1] : ops.k[2]);
+  const int t = blockIdx.x - o.tile0;
+  const int P2 = o.P * o.P, Q2 = o.Q * o.Q;
+  const int i0 = (t / o.tiles_n) * kBT, j0 = (t % o.tiles_n) * kBT;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  double acc[4][4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+#pragma unroll
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
+  for (int r0 = 0; r0 < o.R; r0 += kBK) {
+#pragma unroll
+    for (int q = 0; q < kBK * kBT / 256; ++q) {
+      const int e = threadIdx.x + 256 * q, c = e & (kBT - 1), r = r0 + (e >> 6);
+      As[e >> 6][c] = (r < o.R && i0 + c < P2) ? o.a[(long)r * P2 + i0 + c] : 0.0;
+      Bs[e >> 6][c] = (r < o.R && j0 + c < Q2) ? o.b[(long)r * Q2 + j0 + c] : 0.0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < kBK; ++r) {
+      double a[4], b[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i) a[i] = As[r][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) b[j] = Bs[r][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+    }
+    __syncthreads();
+  }
+  const long PQ = (long)o.P * o.Q;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const int gi = i0 + ty + 16 * i;
+    if (gi >= P2) continue;
+    const int p = gi / o.P, pp = gi % o.P;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const int gj = j0 + tx + 16 * j;
+      if (gj >= Q2) continue;
+      const int q = gj / o.Q, qq = gj % o.Q;
+      double v = acc[i][j];
+      if (o.hp && q == qq) v += o.hp[gi];
+      if (o.hq && p == pp) v += o.hq[gj];
+      o.m[((long)p * o.Q + q) * PQ + (long)pp * o.Q + qq] = v;
+    }
+  }
+}
+
+// ---------------------------------------------------------------- the application
+struct DenseApply {
+  const double* m[3];  // dense operators per pair kind (null: none)
+  const double* x;
+  double* y;
+  int d[3];
+};
+
+__device__ __forceinline__ void cp_async8(uint32_t dst, const double* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(dst), "l"(src) : "memory");
+}
+
+constexpr int kDT = 256;      // threads
+constexpr int kDK = 32;       // K entries per step: one per lane of the loading warps
+constexpr int kDP = kDK + 1;  // padded row: the 32 rows a warp reads lie in different banks
+constexpr int kDStages = 3;
+constexpr int kDFold = 4;
+
+// Shape of pair kind k in a TA x TB x TC block: rows (the block's extent along the pair,
+// second link fastest) and columns (along the remaining link).
+template <int TA, int TB, int TC, int k>
+struct DenseKind {
+  static constexpr int ROWS = k == 0 ? TA * TB : (k == 1 ? TA * TC : TB * TC);
+  static constexpr int INNER = k == 0 ? TB : TC;
+  static constexpr int COLS = k == 0 ? TC : (k == 1 ? TB : TA);
+};
+
+// One CTA: the TA x TB x TC block of y. Each kind is a small GEMM of the block's rows of M
+// with x; blocks of fewer outputs than threads split every K step over G groups of threads,
+// whose sums meet at the end in a fixed order. Each loading warp takes every eighth row, so a
+// thread's rows are one pointer and one stride: with two warps per scheduler the integer work
+// of a step, not its copies, was what a small block waited for (24.6 -> 16.4 us at [16]^3).
+template <int TA, int TB, int TC>
+struct DenseBlock {
+  static constexpr int OUT = TA * TB * TC;
+  static constexpr int G = OUT < kDT ? kDT / OUT : 1;    // thread groups over K
+  static constexpr int PER = OUT < kDT ? 1 : OUT / kDT;  // outputs per thread
+  static constexpr int R01 = TA * TB, R02 = TA * TC, R12 = TB * TC;
+  static constexpr int RMAX = R01 > R02 ? (R01 > R12 ? R01 : R12) : (R02 > R12 ? R02 : R12);
+  static constexpr int CMAX = TA > TB ? (TA > TC ? TA : TC) : (TB > TC ? TB : TC);
+  static constexpr int STAGE = (RMAX + CMAX) * kDP;
+  static_assert(R01 % 8 == 0 && R02 % 8 == 0 && R12 % 8 == 0 && 8 % TB == 0 && 8 % TC == 0 && CMAX <= 8,
+                "eight loading warps share the rows and columns evenly");
+  static_assert(OUT >= kDT ? OUT % kDT == 0 && kDT % R01 == 0 && kDT % R02 == 0 && kDT % R12 == 0 : kDT % OUT == 0,
+                "outputs divide over the threads, with a thread's outputs in one row");
+
+  const DenseApply& g;
+  double* sm;
+  int a0, b0, c0;  // block origin
+  int K[3], n[3];  // reduction lengths and K steps of the kinds (0 steps: no operator)
+  const double* mp[3];  // this thread's first row of M, at its K entry of step 0
+  long mstride[3];      // to its next row (eight rows on)
+  int live[3];          // how many of its rows are inside the tensor
+  double acc[PER], tot[PER];
+
+  __device__ DenseBlock(const DenseApply& g_, double* sm_) : g(g_), sm(sm_) {
+    const int nb1 = (g.d[1] + TB - 1) / TB, nb2 = (g.d[2] + TC - 1) / TC;
+    const int bid = blockIdx.x;
+    a0 = bid / (nb1 * nb2) * TA;
+    b0 = bid / nb2 % nb1 * TB;
+    c0 = bid % nb2 * TC;
+    setup<0>();
+    setup<1>();
+    setup<2>();
+  }
+
+  template <int k>
+  __device__ void setup() {
+    using D = DenseKind<TA, TB, TC, k>;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int outer0 = k == 2 ? b0 : a0, inner0 = k == 0 ? b0 : c0;
+    const int no = k == 2 ? g.d[1] : g.d[0], ni = k == 0 ? g.d[1] : g.d[2];
+    K[k] = no * ni;
+    n[k] = g.m[k] ? (K[k] + kDK - 1) / kDK : 0;
+    const int o = outer0 + w / D::INNER, i = inner0 + w % D::INNER;
+    constexpr int step = 8 / D::INNER;  // links of the outer slot from one row to the next
+    mp[k] = g.m[k] + ((long)o * ni + i) * K[k] + lane;
+    mstride[k] = (long)step * ni * K[k];
+    live[k] = i < ni && o < no ? min(D::ROWS / 8, (no - o + step - 1) / step) : 0;
+  }
+
+  static __device__ __forceinline__ void copy(double* dst, const double* src, bool in) {
+    if (in) cp_async8((uint32_t)__cvta_generic_to_shared(dst), src);
+    else *dst = 0.0;
+  }
+
+  // issue the copies of K step s of kind k into stage st
+  template <int k>
+  __device__ __forceinline__ void load(int s, int st) {
+    using D = DenseKind<TA, TB, TC, k>;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int k0 = s * kDK, kg = k0 + lane;
+    const bool kin = kg < K[k];
+    double* Ms = sm + st * STAGE + w * kDP + lane;
+    const double* src = mp[k] + k0;
+#pragma unroll
+    for (int i = 0; i < D::ROWS / 8; ++i) copy(Ms + 8 * i * kDP, src + i * mstride[k], kin && i < live[k]);
+    double* Xs = sm + st * STAGE + RMAX * kDP;
+    const int m1 = g.d[1], m2 = g.d[2];
+    if (k == 0) {  // x[k][c]: contiguous along the columns
+#pragma unroll
+      for (int e = threadIdx.x; e < D::COLS * kDK; e += kDT) {
+        const int c = e % TC, kk = e / TC, ke = k0 + kk;
+        copy(Xs + c * kDP + kk, g.x + (long)ke * m2 + c0 + c, ke < K[0] && c0 + c < m2);
+      }
+    } else if (w < D::COLS) {
+      if (k == 1) {
+        const unsigned kp = (unsigned)kg / (unsigned)m2, kc = (unsigned)kg - kp * (unsigned)m2;
+        copy(Xs + w * kDP + lane, g.x + ((long)kp * m1 + b0 + w) * m2 + kc, kin && b0 + w < m1);
+      } else {
+        copy(Xs + w * kDP + lane, g.x + (long)(a0 + w) * K[2] + kg, kin && a0 + w < g.d[0]);
+      }
+    }
+  }
+  // step `at` of the three kinds' steps in a row
+  __device__ __forceinline__ void issue(int at, int st) {
+    if (at < n[0]) load<0>(at, st);
+    else if (at < n[0] + n[1]) load<1>(at - n[0], st);
+    else if (at < n[0] + n[1] + n[2]) load<2>(at - n[0] - n[1], st);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+
+  // all steps of kind k, the first being step `at` of the whole; adds its outputs to ysum
+  template <int k>
+  __device__ __forceinline__ void run(int& at, int& st, double* ysum) {
+    using D = DenseKind<TA, TB, TC, k>;
+    const int grp = G > 1 ? threadIdx.x / OUT : 0, o = G > 1 ? threadIdx.x % OUT : threadIdx.x;
+    const int row = o % D::ROWS, col = o / D::ROWS;
+    constexpr int CSTEP = PER > 1 ? kDT / D::ROWS : 0;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) acc[j] = tot[j] = 0.0;
+    for (int s = 0; s < n[k]; ++s, ++at) {
+      asm volatile("cp.async.wait_group %0;" ::"n"(kDStages - 2) : "memory");
+      __syncthreads();
+      issue(at + kDStages - 1, st == 0 ? kDStages - 1 : st - 1);
+      const double* mr = sm + st * STAGE + row * kDP + grp;
+      const double* xc = sm + st * STAGE + RMAX * kDP + col * kDP + grp;
+#pragma unroll
+      for (int q = 0; q < kDK; q += G) {
+        const double mv = mr[q];
+#pragma unroll
+        for (int j = 0; j < PER; ++j) acc[j] = fma(mv, xc[j * CSTEP * kDP + q], acc[j]);
+      }
+      // sums run over kDFold K steps before they join the total, so that rounding grows with
+      // the root of that many terms and not of the whole row of M
+      if (s % kDFold == kDFold - 1) {
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+          tot[j] += acc[j];
+          acc[j] = 0.0;
+        }
+      }
+      st = st == kDStages - 1 ? 0 : st + 1;
+    }
+    if (n[k] == 0) return;
+#pragma unroll
+    for (int j = 0; j < PER; ++j) {
+      const int cj = col + j * CSTEP, ro = row / D::INNER, ri = row % D::INNER;
+      const int a = k == 2 ? cj : ro, b = k == 0 ? ri : (k == 1 ? cj : ro), c = k == 0 ? cj : ri;
+      ysum[grp * OUT + (a * TB + b) * TC + c] += tot[j] + acc[j];
+    }
+    __syncthreads();  // the next kind's outputs belong to other threads
+  }
+};
+
+template <int TA, int TB, int TC>
+__global__ void __launch_bounds__(kDT) dense_apply_kernel(const __grid_constant__ DenseApply g) {
+  using B = DenseBlock<TA, TB, TC>;
+  extern __shared__ double sm[];
+  double* ysum = sm + kDStages * B::STAGE;  // [G][OUT]
+  B blk(g, sm);
+  for (int e = threadIdx.x; e < B::G * B::OUT; e += kDT) ysum[e] = 0.0;
+#pragma unroll
+  for (int i = 0; i < kDStages - 1; ++i) blk.issue(i, i);
+  int at = 0, st = 0;
+  blk.template run<0>(at, st, ysum);
+  blk.template run<1>(at, st, ysum);
+  blk.template run<2>(at, st, ysum);
+  __syncthreads();
+  for (int o = threadIdx.x; o < B::OUT; o += kDT) {
+    double v = ysum[o];
+#pragma unroll
+    for (int q = 1; q < B::G; ++q) v += ysum[q * B::OUT + o];
+    const int a = blk.a0 + o / (TB * TC), b = blk.b0 + o / TC % TB, c = blk.c0 + o % TC;
+    if (a < g.d[0] && b < g.d[1] && c < g.d[2]) g.y[((long)a * g.d[1] + b) * g.d[2] + c] = v;
+  }
+}
+
+template <int TA, int TB, int TC>
+void launch_dense(cudaStream_t st, const DenseApply& g) {
+  using B = DenseBlock<TA, TB, TC>;
+  constexpr size_t smem = sizeof(double) * (kDStages * B::STAGE + B::G * B::OUT);
+  static bool attr = false;  // (set again by a second thread: harmless)
+  if (!attr) {
+    ATTN_CHECK_CUDA(cudaFuncSetAttribute(dense_apply_kernel<TA, TB, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem));
+    attr = true;
+  }
+  const long blocks = (long)((g.d[0] + TA - 1) / TA) * ((g.d[1] + TB - 1) / TB) * ((g.d[2] + TC - 1) / TC);
+  dense_apply_kernel<TA, TB, TC><<<(unsigned)blocks, kDT, smem, st>>>(g);
+}
+
+// What the choices below weigh: the FP64 FMA rate that the kernels reach, a dependent launch
+// and a device allocation (measured: 1.11 TFLOP/s at [64]^3, about 4 us and 50 us).
+constexpr double kF64Rate = 1.1e12, kLaunch = 4e-6, kAlloc = 5e-5;
+
+}  // namespace
+
+// Device memory for dense operators: at most a sixteenth of the GPU per context and, for more
+// than 64 MB at once, at most a quarter of what is free, so that programs with many handles or
+// a pool of their own keep the product-by-product path instead of running out. False when
+// there is no room (buf is then empty and no longer counted).
+bool dense_reserve(attn_ctx* ctx, DevBuf& buf, size_t n, size_t& counted) {
+  if (n <= buf.bytes) return true;
+  bool ok = ctx->dense_bytes - counted + n <= ctx->total_mem / 16;
+  if (ok && n > (64u << 20)) {
+    size_t fr = 0, total = 0;
+    ok = cudaMemGetInfo(&fr, &total) == cudaSuccess && n <= fr / 4 + buf.bytes;
+    (void)cudaGetLastError();
+  }
+  if (!ok) return false;
+  ctx->dense_bytes -= counted;
+  counted = 0;
+  try {
+    buf.reserve(n);
+  } catch (const Error& e) {
+    if (e.status != ATTN_ENOMEM) throw;
+    return false;
+  }
+  counted = buf.bytes;
+  ctx->dense_bytes += counted;
+  return true;
+}
+
+bool stream_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &cs) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return true;
+  }
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+DenseF64::~DenseF64() {
+  if (ctx) ctx->dense_bytes -= bytes;
+}
+
+// Which pair kinds are worth a dense operator for `uses` applications, and whether making
+// them pays. Per kind: (PQ)^2 S against R (P + Q) PQ S operations, and the launches of the
+// product path (per kind a mode product, a sum over products and its split, and a share of
+// the fill and the internal operators).
+static bool plan_dense(const attn_heff* h, double uses, bool (&use)[3]) {
+  // a handle's first dense operators also cost an allocation
+  double gain = 0.0, build = kLaunch + (h->dense ? 0.0 : kAlloc);
+  bool any = false;
+  for (int k = 0; k < 3; ++k) {
+    const double P = h->m[kPairP[k]], Q = h->m[kPairQ[k]], S = h->m[kPairS[k]], R = h->npair[k];
+    use[k] = false;
+    if (h->npair[k] == 0) continue;
+    const double direct = 2.0 * R * (P + Q) * P * Q * S / kF64Rate + 5 * kLaunch;
+    const double dense = 2.0 * P * Q * P * Q * S / kF64Rate;
+    const double make = 2.0 * R * P * P * Q * Q / kF64Rate;
+    if (dense >= direct) continue;
+    use[k] = true;
+    any = true;
+    gain += direct - dense;
+    build += make;
+  }
+  return any && uses * gain >= build;
+}
+
+void dense_invalidate(attn_heff* h) {
+  if (h->dense) h->dense->ready = false;
+  h->f64_uses = 0;
+  h->expect = 1;
+}
+
+void dense_release(attn_heff* h) {
+  delete h->dense;
+  h->dense = nullptr;
+}
+
+// The dense FP64 operators of h, made when they pay for the applications so far plus the
+// ones announced (h->expect); null when the product-by-product path is the cheaper one.
+DenseF64* dense_f64(attn_heff* h) {
+  attn_ctx* ctx = h->ctx;
+  if (h->dense && h->dense->ready) return h->dense;
+  // an application counts for itself and for those already made: a caller who comes back
+  // will come back again
+  const double uses = std::max<double>(h->expect, h->f64_uses > 0 ? 1 + 4.0 * h->f64_uses : 1.0);
+  ++h->f64_uses;
+  bool use[3];
+  if (!plan_dense(h, uses, use) || stream_capturing(ctx->stream)) return nullptr;
+  if (!h->dense) h->dense = new DenseF64();
+  DenseF64* d = h->dense;
+  d->ctx = ctx;
+  size_t need = 0;
+  for (int k = 0; k < 3; ++k) {
+    const size_t pq = (size_t)h->m[kPairP[k]] * h->m[kPairQ[k]];
+    d->at[k] = need;
+    if (use[k]) need += pq * pq;
+  }
+  if (!dense_reserve(ctx, d->buf, sizeof(double) * need, d->bytes)) return nullptr;
+  PairOps ops;
+  ops.n = 0;
+  int tiles = 0;
+  bool hint_done[3] = {false, false, false};
+  for (int k = 0; k < 3; ++k) {
+    d->use[k] = use[k];
+    if (!use[k]) continue;
+    const int p = kPairP[k], q = kPairQ[k];
+    PairOp& o = ops.k[ops.n++];
+    o.P = h->m[p];
+    o.Q = h->m[q];
+    o.R = h->npair[k];
+    o.a = h->pa[k].as<double>();
+    o.b = h->pb[k].as<double>();
+    o.m = d->m(k);
+    // an internal operator joins the first dense kind that acts on its link
+    o.hp = h->has_hint[p] && !hint_done[p] ? h->hint[p].as<double>() : nullptr;
+    o.hq = h->has_hint[q] && !hint_done[q] ? h->hint[q].as<double>() : nullptr;
+    hint_done[p] = hint_done[q] = true;
+    o.tiles_n = (o.Q * o.Q + kBT - 1) / kBT;
+    o.tile0 = tiles;
+    tiles += o.tiles_n * ((o.P * o.P + kBT - 1) / kBT);
+  }
+  for (int s = 0; s < 3; ++s) d->hint[s] = hint_done[s];
+  pair_operator_kernel<<<tiles, 256, 0, ctx->stream>>>(ops);
+  ctx->launches++;
+  ATTN_CHECK_CUDA(cudaGetLastError());
+  d->ready = true;
+  return d;
+}
+
+// y = (dense kinds) x; every entry of y is written.
+void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y) {
+  attn_ctx* ctx = h->ctx;
+  DenseApply g;
+  double fl = 0.0;
+  for (int k = 0; k < 3; ++k) {
+    g.m[k] = d->use[k] ? d->m(k) : nullptr;
+    const double pq = (double)h->m[kPairP[k]] * h->m[kPairQ[k]];
+    if (d->use[k]) fl += 2.0 * pq * pq * h->m[kPairS[k]];
+    g.d[k] = h->m[k];
+  }
+  g.x = x;
+  g.y = y;
+  // Block of y by the outputs that the busiest SM computes (FP64 FMAs bound the kernel),
+  // weighted by what a block shape loses to its loads; measured at 8 to 96 on all links, where
+  // the rule takes the fastest shape or one within 3 % of it.
+  const long sms = std::max(ctx->num_sms, 1);
+  const int* m = h->m;
+  auto cost = [&](int ta, int tb, int tc, double weight) {
+    const long blocks = (long)((m[0] + ta - 1) / ta) * ((m[1] + tb - 1) / tb) * ((m[2] + tc - 1) / tc);
+    return weight * (double)((blocks + sms - 1) / sms * (ta * tb * tc));
+  };
+  const double c[5] = {cost(8, 8, 8, 1.0), cost(4, 8, 8, 1.0), cost(4, 4, 8, 1.02), cost(4, 4, 4, 1.1),
+                       cost(4, 4, 2, 1.28)};
+  const int best = (int)(std::min_element(c, c + 5) - c);
+  ctx->prof_begin(1);
+  if (best == 0) launch_dense<8, 8, 8>(ctx->stream, g);
+  else if (best == 1) launch_dense<4, 8, 8>(ctx->stream, g);
+  else if (best == 2) launch_dense<4, 4, 8>(ctx->stream, g);
+  else if (best == 3) launch_dense<4, 4, 4>(ctx->stream, g);
+  else launch_dense<4, 4, 2>(ctx->stream, g);
+  ctx->prof_end(1, fl);
+  ctx->launches++;
+  ATTN_CHECK_CUDA(cudaGetLastError());
+}
+
+}  // namespace attn

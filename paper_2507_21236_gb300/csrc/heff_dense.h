@@ -1,0 +1,33 @@
+// One dense operator per link pair of an effective Hamiltonian (internal).
+#pragma once
+
+#include "attn_internal.h"
+
+struct attn_heff;
+
+namespace attn {
+
+// FP64 operators M_k [P Q][P Q] of the pair kinds whose products are summed (use[k]), one
+// after another in one buffer; hint[s]: the internal operator of slot s is part of one of them.
+struct DenseF64 {
+  attn_ctx* ctx = nullptr;
+  DevBuf buf;
+  size_t at[3] = {0, 0, 0};
+  double* m(int k) const { return buf.as<double>() + at[k]; }
+  bool use[3] = {false, false, false}, hint[3] = {false, false, false};
+  bool ready = false;
+  size_t bytes = 0;  // counted in ctx->dense_bytes
+  ~DenseF64();
+};
+
+// buf of at least n bytes within the context's share of device memory for dense operators;
+// `counted` is what buf has in that count.
+bool dense_reserve(attn_ctx* ctx, DevBuf& buf, size_t n, size_t& counted);
+bool stream_capturing(cudaStream_t st);
+
+DenseF64* dense_f64(attn_heff* h);
+void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y);
+void dense_invalidate(attn_heff* h);
+void dense_release(attn_heff* h);
+
+}  // namespace attn

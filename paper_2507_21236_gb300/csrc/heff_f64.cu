@@ -5,7 +5,8 @@
 // Each product group is two (three for triples) strided GEMM stages: stage 1
 // applies the second operator of every product of a chunk to x, writing one
 // intermediate per product; stage 2 is a single GEMM whose reduction runs over
-// (product, link index), accumulating straight into y.
+// (product, link index), accumulating straight into y. Pair kinds with enough products
+// go through their sum instead (heff_dense.cu).
 #include <algorithm>
 
 #include "heff.h"
@@ -24,6 +25,7 @@ double attn_heff::flops() const {
 attn_heff::~attn_heff() {
   delete eg;
   attn::tc_release(this);
+  attn::dense_release(this);
 }
 
 namespace attn {
@@ -59,14 +61,17 @@ void accumulate_slot_f64(attn_ctx* ctx, const int d[3], int p, const double* A, 
 
 void attn_heff::apply_f64(const double* x, double* y) {
   const int d[3] = {m[0], m[1], m[2]};
-  fill_f64(ctx, y, (size_t)V, 0.0);
+  const DenseF64* dn = ctx->cfg.f64_split ? nullptr : dense_f64(this);
+  if (dn) dense_apply_f64(this, dn, x, y);
+  else fill_f64(ctx, y, (size_t)V, 0.0);
   for (int s = 0; s < 3; ++s)
-    if (has_hint[s]) mode_product_f64(ctx, d, s, hint[s].as<double>(), 1, x, 0, y, 1.0);
+    if (has_hint[s] && !(dn && dn->hint[s])) mode_product_f64(ctx, d, s, hint[s].as<double>(), 1, x, 0, y, 1.0);
   // chunk so that the intermediates stay below ~1 GiB
   const long budget = 1L << 27;  // doubles
   const int chunk = (int)std::max<long>(1, std::min<long>(4096, budget / std::max<long>(V, 1)));
   for (int k = 0; k < 3; ++k) {
     const int p = kPairP[k], q = kPairQ[k];
+    if (dn && dn->use[k]) continue;
     for (int r0 = 0; r0 < npair[k]; r0 += chunk) {
       const int R = std::min(chunk, npair[k] - r0);
       ctx->ws[0].reserve(sizeof(double) * (size_t)R * V);

@@ -358,6 +358,7 @@ void attn_state::recycle(attn_heff* h) {
   delete h->eg;  // a captured graph holds the old operators' launch parameters
   h->eg = nullptr;
   attn::tc_invalidate(h);
+  attn::dense_invalidate(h);
   spare_heff = h;
 }
 
@@ -469,6 +470,8 @@ double attn_state::local_step(int n) {
     const attn_dtype dt = (cfg.matvec_dtype != ATTN_F64 && tc_supported(h)) ? cfg.matvec_dtype : ATTN_F64;
     MatVec mv_lo = [&](const double* a, double* b) { h->apply(a, b, dt); };
     MatVec mv64 = [&](const double* a, double* b) { h->apply_f64(a, b); };
+    // FP64 applications to come: the Krylov depth, or one per correction
+    h->expect = dt == ATTN_F64 ? cfg.lanczos_depth : 1 + std::max(cfg.refine_steps, 0);
     // current energy (FP64): known from the last local step unless H' or a tensor changed since
     double e_cur = energy_known;
     if (!std::isfinite(e_cur)) {
