@@ -51,7 +51,8 @@ struct attn_heff {
   // FP64 operators summed per link pair, once they pay (heff_dense.cu): applications made,
   // and how many the caller of the next ones announces (a Lanczos its depth)
   attn::DenseF64* dense = nullptr;
-  int f64_uses = 0, expect = 1;
+  attn::DenseSplit* dense_s = nullptr;  // the same as BF16 slices (f64_split)
+  int f64_uses = 0, split_uses = 0, expect = 1;
   EigGraph* eg = nullptr; // cached eigensolve graph (use_graphs)
   attn::DevBuf host_x;    // device copy of the tensor of attn_eigsolve_host
   double flops() const;

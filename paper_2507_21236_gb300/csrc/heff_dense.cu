@@ -11,13 +11,21 @@
 // FP64 on the CUDA cores. This GPU executes two FP64 FMAs per SM and cycle, so the number of
 // FMAs decides (M streams from L2 or HBM far below their rates), and a simple kernel saturates
 // it: every CTA owns a block of y and adds the contributions of all three pair kinds to it,
-// in a fixed order, with no workspace and no second launch. Measured (GB300, one
+// in a fixed order, with no workspace and no second launch.
+//
+// With f64_split, M is held as its six BF16 slices (12 bytes per entry, written once), and an
+// application is one split GEMM per kind instead of two with a 1 GiB intermediate that has to be
+// sliced in between. Measured (GB300, one
 // application): [64]^3 with 140 products per pair 25.4 -> 5.6 ms; [16]^3 with 12
-// 128 -> 16 us, where the product-by-product path spends its time on 17 launches.
+// 128 -> 16 us, where the product-by-product path spends its time on 17 launches; f64_split at
+// [128]^3 with 288: 42.3 -> 3.5 ms (first application, which makes the slices: 42.7 -> 23.7 ms),
+// error against 64 bits 1.1e-13 -> 7.7e-14.
 #include <algorithm>
+#include <cmath>
 
 #include "heff.h"
 #include "heff_dense.h"
+#include "ozaki.h"
 
 namespace attn {
 
@@ -344,6 +352,9 @@ bool stream_capturing(cudaStream_t st) {
 DenseF64::~DenseF64() {
   if (ctx) ctx->dense_bytes -= bytes;
 }
+DenseSplit::~DenseSplit() {
+  if (ctx) ctx->dense_bytes -= bytes;
+}
 
 // Which pair kinds are worth a dense operator for `uses` applications, and whether making
 // them pays. Per kind: (PQ)^2 S against R (P + Q) PQ S operations, and the launches of the
@@ -371,13 +382,16 @@ static bool plan_dense(const attn_heff* h, double uses, bool (&use)[3]) {
 
 void dense_invalidate(attn_heff* h) {
   if (h->dense) h->dense->ready = false;
-  h->f64_uses = 0;
+  if (h->dense_s) h->dense_s->ready = false;
+  h->f64_uses = h->split_uses = 0;
   h->expect = 1;
 }
 
 void dense_release(attn_heff* h) {
   delete h->dense;
+  delete h->dense_s;
   h->dense = nullptr;
+  h->dense_s = nullptr;
 }
 
 // The dense FP64 operators of h, made when they pay for the applications so far plus the
@@ -464,6 +478,185 @@ void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y
   else if (best == 3) launch_dense<4, 4, 4>(ctx->stream, g);
   else launch_dense<4, 4, 2>(ctx->stream, g);
   ctx->prof_end(1, fl);
+  ctx->launches++;
+  ATTN_CHECK_CUDA(cudaGetLastError());
+}
+
+// ---------------------------------------------------------------- as BF16 slices
+namespace {
+
+// M += H_p (x) 1 and 1 (x) H_q (either may be null) on the rows (i, j), i0 <= i < i1, that m
+// holds; one thread per row, since both add to the row's diagonal entry.
+__global__ void add_internal_kernel(double* m, int P, int Q, int i0, int i1, const double* hp, const double* hq) {
+  const long PQ = (long)P * Q;
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)(i1 - i0) * Q; e += (long)gridDim.x * blockDim.x) {
+    const int i = i0 + (int)(e / Q), j = (int)(e % Q);
+    double* row = m + e * PQ;
+    if (hp)
+      for (int ii = 0; ii < P; ++ii) row[(long)ii * Q + j] += hp[(long)i * P + ii];
+    if (hq)
+      for (int jj = 0; jj < Q; ++jj) row[(long)i * Q + jj] += hq[(long)j * Q + jj];
+  }
+}
+
+// y[a][b][c] = sum over the K parts of the kinds' outputs P01[c][(a, b)], P02[b][(a, c)],
+// P12[a][(b, c)], in that order; 32 x 32 tiles of the (b, c) plane, the first through shared memory.
+struct SplitParts {
+  const double* p[3];
+  int n[3];
+};
+__global__ void split_combine_kernel(double* __restrict__ y, int m0, int m1, int m2, const SplitParts s) {
+  __shared__ double t[32][33];
+  const long V = (long)m0 * m1 * m2;
+  const int a = blockIdx.z, b0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
+  auto sum = [&](const double* p, int n, long at) {
+    double v = p[at];
+    for (int i = 1; i < n; ++i) v += p[at + i * V];
+    return v;
+  };
+  if (s.n[0]) {
+    for (int cc = threadIdx.y; cc < 32; cc += blockDim.y) {
+      const int c = c0 + cc, b = b0 + threadIdx.x;
+      if (b < m1 && c < m2) t[threadIdx.x][cc] = sum(s.p[0], s.n[0], ((long)c * m0 + a) * m1 + b);
+    }
+    __syncthreads();
+  }
+  for (int bb = threadIdx.y; bb < 32; bb += blockDim.y) {
+    const int b = b0 + bb, c = c0 + threadIdx.x;
+    if (b < m1 && c < m2) {
+      double v = s.n[0] ? t[bb][threadIdx.x] : 0.0;
+      if (s.n[1]) v += sum(s.p[1], s.n[1], ((long)b * m0 + a) * m2 + c);
+      if (s.n[2]) v += sum(s.p[2], s.n[2], ((long)a * m1 + b) * m2 + c);
+      y[((long)a * m1 + b) * m2 + c] = v;
+    }
+  }
+}
+
+// Times of the split path on this GPU (measured at 64 and 128 on all links): product by product
+// 25 ps per intermediate entry and product (both GEMM stages, exponents and slicing of the
+// intermediate), slices of M 20 ps per entry to make, 1.4 ps per entry and 64 slices to apply,
+// and the launches of a kind; FP64 FMAs as above.
+constexpr double kSplitProd = 25e-12, kSplitMake = 20e-12, kSplitUse = 1.4e-12, kSplitKind = 5e-5;
+constexpr long kStage = 1L << 27;  // doubles of M made at a time (1 GiB)
+
+}  // namespace
+
+DenseSplit* dense_split(attn_heff* h) {
+  attn_ctx* ctx = h->ctx;
+  if (h->dense_s && h->dense_s->ready) return h->dense_s;
+  const double uses = std::max<double>(h->expect, h->split_uses > 0 ? 1 + 4.0 * h->split_uses : 1.0);
+  ++h->split_uses;
+  bool use[3], any = false;
+  double gain = 0.0, build = 2e-4;  // and two allocations
+  size_t need = 0, ne = 0, at[3], eat[3];
+  int kpart[3] = {0, 0, 0};
+  for (int k = 0; k < 3; ++k) {
+    const double P = h->m[kPairP[k]], Q = h->m[kPairQ[k]], S = h->m[kPairS[k]], R = h->npair[k];
+    const double direct = R * h->V * kSplitProd + kSplitKind;
+    const double dense = P * Q * P * Q * std::ceil(S / 64.0) * kSplitUse + kSplitKind;
+    at[k] = need;
+    eat[k] = ne;
+    // (a slice row has at most 65536 entries: the int64 sums of the split GEMM)
+    use[k] = h->npair[k] > 0 && 2.0 * dense < direct && P * Q <= 65536.0 && P >= 16 && Q >= 16;
+    if (!use[k]) continue;
+    any = true;
+    gain += direct - dense;
+    build += P * Q * P * Q * kSplitMake * (1.0 + R / 600.0);
+    const long pq = (long)P * (long)Q;
+    kpart[k] = oz_kparts((int)pq, (int)S, pq, std::max(ctx->num_sms, 1));
+    const long parts = (pq + kpart[k] - 1) / kpart[k];
+    need += ozaki_slice_bytes(parts, pq, kpart[k], 128);
+    ne += (size_t)(parts * pq);
+  }
+  if (!any || uses * gain < build || stream_capturing(ctx->stream)) return nullptr;
+  if (!h->dense_s) h->dense_s = new DenseSplit();
+  DenseSplit* d = h->dense_s;
+  d->ctx = ctx;
+  if (!dense_reserve(ctx, d->slices, need, d->bytes)) return nullptr;
+  d->exps.reserve(sizeof(int) * ne);
+  bool hint_done[3] = {false, false, false};
+  for (int k = 0; k < 3; ++k) {
+    d->use[k] = use[k];
+    d->at[k] = at[k];
+    d->eat[k] = eat[k];
+    d->kpart[k] = kpart[k];
+    if (!use[k]) continue;
+    const int p = kPairP[k], q = kPairQ[k], P = h->m[p], Q = h->m[q], R = h->npair[k];
+    const long PQ = (long)P * Q, parts = (PQ + kpart[k] - 1) / kpart[k], tiles = (PQ + 127) / 128;
+    const long part_slices = tiles * (kpart[k] / 64) * 6 * 128 * 64;
+    const double* hp = h->has_hint[p] && !hint_done[p] ? h->hint[p].as<double>() : nullptr;
+    const double* hq = h->has_hint[q] && !hint_done[q] ? h->hint[q].as<double>() : nullptr;
+    hint_done[p] = hint_done[q] = true;
+    // values of the first link at a time: whole 128-row tiles of M, about kStage entries
+    int unit = 1;
+    while (unit < 128 && (unit * Q) % 128) ++unit;
+    const int step = (int)std::max<long>(1, std::min<long>(P, kStage / (PQ * Q)) / unit) * unit;
+    ctx->ws[0].reserve(sizeof(double) * (size_t)std::min(step, P) * Q * PQ);
+    double* stage = ctx->ws[0].as<double>();
+    for (int i0 = 0; i0 < P; i0 += step) {
+      const int i1 = std::min(P, i0 + step);
+      GemmF64 g;  // M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j'], a batch entry per (i, j)
+      g.split_ok = true;
+      g.M = P; g.N = Q; g.K = R;
+      g.Bhi = i1 - i0; g.Blo = Q;
+      g.A = h->pa[k].as<double>() + (long)i0 * P; g.aM = 1; g.aK = (long)P * P; g.aBhi = P;
+      g.B = h->pb[k].as<double>(); g.bN = 1; g.bK = (long)Q * Q; g.bBlo = Q;
+      g.C = stage; g.cM = Q; g.cN = 1; g.cBhi = Q * PQ; g.cBlo = PQ;
+      gemm_f64(ctx, g);
+      if (hp || hq) {
+        const long rows = (long)(i1 - i0) * Q;
+        add_internal_kernel<<<(int)std::min<long>((rows + 127) / 128, 4096), 128, 0, ctx->stream>>>(stage, P, Q, i0, i1,
+                                                                                                hp, hq);
+        ctx->launches++;
+      }
+      OzView v;
+      v.p = stage;
+      v.sR = PQ; v.sK = 1;
+      v.rows = (int)((i1 - i0) * Q);
+      v.K = (int)PQ;
+      v.kpart = kpart[k];
+      const long row0 = (long)i0 * Q;
+      auto* s = reinterpret_cast<__nv_bfloat16*>(d->slices.as<uint8_t>() + at[k]) +
+                row0 / 128 * (kpart[k] / 64) * 6 * 128 * 64;
+      v.nblo = (int)parts;
+      ozaki_slice_to(ctx, v, kpart[k], 128, s, d->exps.as<int>() + eat[k] + row0, part_slices, PQ);
+    }
+  }
+  for (int s = 0; s < 3; ++s) d->hint[s] = hint_done[s];
+  ATTN_CHECK_CUDA(cudaGetLastError());
+  d->ready = true;
+  return d;
+}
+
+void dense_apply_split(attn_heff* h, const DenseSplit* d, const double* x, double* y) {
+  attn_ctx* ctx = h->ctx;
+  const int m0 = h->m[0], m1 = h->m[1], m2 = h->m[2];
+  SplitParts parts;
+  size_t total = 0, off[3];
+  for (int k = 0; k < 3; ++k) {
+    const long pq = (long)h->m[kPairP[k]] * h->m[kPairQ[k]];
+    parts.n[k] = d->use[k] ? (int)((pq + d->kpart[k] - 1) / d->kpart[k]) : 0;
+    off[k] = total;
+    total += (size_t)parts.n[k] * h->V;
+  }
+  ctx->ws[0].reserve(sizeof(double) * total);
+  for (int k = 0; k < 3; ++k) {
+    parts.p[k] = ctx->ws[0].as<double>() + off[k];
+    if (!d->use[k]) continue;
+    OzView q;  // x as [slice][K]: the slices of kind k along its third link
+    q.p = x;
+    q.rows = h->m[kPairS[k]];
+    if (k == 0) { q.sR = 1; q.sK = m2; q.K = m0 * m1; }
+    else if (k == 1) { q.sR = m2; q.sK = 1; q.K = m2; q.G = m0; q.sG = (long)m1 * m2; }
+    else { q.sR = (long)m1 * m2; q.sK = 1; q.K = m1 * m2; }
+    q.kpart = d->kpart[k];
+    q.nblo = parts.n[k];
+    const long pq = (long)h->m[kPairP[k]] * h->m[kPairQ[k]];
+    gemm_f64_presliced(ctx, reinterpret_cast<const __nv_bfloat16*>(d->slices.as<uint8_t>() + d->at[k]),
+                       d->exps.as<int>() + d->eat[k], (int)pq, q, ctx->ws[0].as<double>() + off[k]);
+  }
+  dim3 grid((m2 + 31) / 32, (m1 + 31) / 32, m0);
+  split_combine_kernel<<<grid, dim3(32, 8), 0, ctx->stream>>>(y, m0, m1, m2, parts);
   ctx->launches++;
   ATTN_CHECK_CUDA(cudaGetLastError());
 }

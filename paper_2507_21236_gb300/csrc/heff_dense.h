@@ -20,6 +20,19 @@ struct DenseF64 {
   ~DenseF64();
 };
 
+// The same operators as BF16 slices (ozaki.h) for applications with f64_split: six slices of each
+// M_k in 128-row tiles and the row exponents, one kind after another.
+struct DenseSplit {
+  attn_ctx* ctx = nullptr;
+  DevBuf slices, exps;
+  size_t at[3] = {0, 0, 0}, eat[3] = {0, 0, 0};  // first slice byte and exponent of each kind
+  int kpart[3] = {0, 0, 0};                      // entries of a row that share an exponent
+  bool use[3] = {false, false, false}, hint[3] = {false, false, false};
+  bool ready = false;
+  size_t bytes = 0;
+  ~DenseSplit();
+};
+
 // buf of at least n bytes within the context's share of device memory for dense operators;
 // `counted` is what buf has in that count.
 bool dense_reserve(attn_ctx* ctx, DevBuf& buf, size_t n, size_t& counted);
@@ -27,6 +40,9 @@ bool stream_capturing(cudaStream_t st);
 
 DenseF64* dense_f64(attn_heff* h);
 void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y);
+// The slices, made when they pay; null when products (or FP64 FMAs) are the faster way.
+DenseSplit* dense_split(attn_heff* h);
+void dense_apply_split(attn_heff* h, const DenseSplit* d, const double* x, double* y);
 void dense_invalidate(attn_heff* h);
 void dense_release(attn_heff* h);
 

@@ -61,17 +61,39 @@ void accumulate_slot_f64(attn_ctx* ctx, const int d[3], int p, const double* A, 
 
 void attn_heff::apply_f64(const double* x, double* y) {
   const int d[3] = {m[0], m[1], m[2]};
-  const DenseF64* dn = ctx->cfg.f64_split ? nullptr : dense_f64(this);
-  if (dn) dense_apply_f64(this, dn, x, y);
-  else fill_f64(ctx, y, (size_t)V, 0.0);
+  // pair kinds (and internal operators) that go through their sum: all of y is written
+  bool done[3] = {false, false, false}, hdone[3] = {false, false, false};
+  auto take = [&](const auto* dn) {
+    for (int k = 0; k < 3; ++k) {
+      done[k] = dn->use[k];
+      hdone[k] = dn->hint[k];
+    }
+  };
+  const DenseSplit* ds = ctx->cfg.f64_split ? dense_split(this) : nullptr;
+  // a node too small for slice products (gemm_f64) runs on FP64 FMAs with f64_split as well
+  bool fma = !ctx->cfg.f64_split;
+  if (!fma && !ds) {
+    fma = true;
+    for (int k = 0; k < 3; ++k) fma = fma && 2.0 * npair[k] * V * std::max(m[kPairP[k]], m[kPairQ[k]]) < 1e8;
+  }
+  const DenseF64* dn = fma ? dense_f64(this) : nullptr;
+  if (ds) {
+    dense_apply_split(this, ds, x, y);
+    take(ds);
+  } else if (dn) {
+    dense_apply_f64(this, dn, x, y);
+    take(dn);
+  } else {
+    fill_f64(ctx, y, (size_t)V, 0.0);
+  }
   for (int s = 0; s < 3; ++s)
-    if (has_hint[s] && !(dn && dn->hint[s])) mode_product_f64(ctx, d, s, hint[s].as<double>(), 1, x, 0, y, 1.0);
+    if (has_hint[s] && !hdone[s]) mode_product_f64(ctx, d, s, hint[s].as<double>(), 1, x, 0, y, 1.0);
   // chunk so that the intermediates stay below ~1 GiB
   const long budget = 1L << 27;  // doubles
   const int chunk = (int)std::max<long>(1, std::min<long>(4096, budget / std::max<long>(V, 1)));
   for (int k = 0; k < 3; ++k) {
     const int p = kPairP[k], q = kPairQ[k];
-    if (dn && dn->use[k]) continue;
+    if (done[k]) continue;
     for (int r0 = 0; r0 < npair[k]; r0 += chunk) {
       const int R = std::min(chunk, npair[k] - r0);
       ctx->ws[0].reserve(sizeof(double) * (size_t)R * V);

@@ -401,6 +401,14 @@ __global__ void __launch_bounds__(kOzThreads, 1) ozaki_gemm_kernel(const __grid_
 
 // ------------------------------------------------------------ slicing kernels
 // Operand element (batch bh, bl; row r; k' = g K + k) of a strided FP64 view.
+// First k' of batch entry bl and how many it has (the whole of K', or one of its parts).
+__device__ __forceinline__ long oz_kbase(const OzView& v, int bl) { return v.kpart ? (long)bl * v.kpart : 0; }
+__device__ __forceinline__ long oz_kcount(const OzView& v, int bl) {
+  const long Kt = (long)v.K * v.G;
+  if (!v.kpart) return Kt;
+  const long left = Kt - (long)bl * v.kpart;
+  return left < v.kpart ? left : v.kpart;
+}
 __device__ __forceinline__ long oz_offset(const OzView& v, int bh, int bl, long r, long kk) {
   const long g = kk / v.K, k = kk - g * v.K;
   return (long)bh * v.sBhi + (long)bl * v.sBlo + r * v.sR + g * v.sG + k * v.sK;
@@ -408,8 +416,10 @@ __device__ __forceinline__ long oz_offset(const OzView& v, int bh, int bl, long 
 
 constexpr int kT = 32;  // 32 rows x 32 k per tile, 32 x 8 threads
 
-__global__ void fill_int_kernel(int* p, long n, int v) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) p[i] = v;
+// p[b][r] = v for r < rows of nb batch entries `stride` apart
+__global__ void fill_int_kernel(int* p, long nb, long rows, long stride, int v) {
+  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < nb * rows; i += (long)gridDim.x * blockDim.x)
+    p[i / rows * stride + i % rows] = v;
 }
 
 // Binary exponent e of a finite nonzero double (|x| = f 2^e, f in [0.5, 1)) from its
@@ -424,12 +434,12 @@ __device__ __forceinline__ int exp_bits(long long b) {
 // E[batch][row] = max over k' of the binary exponent of |entry| (|entry| < 2^E).
 // Lanes walk k when k is the unit stride (each warp then owns four rows of the
 // tile), rows otherwise; every shuffle runs on the whole warp.
-__global__ void oz_exponent_kernel(OzView v, int* E) {
+__global__ void oz_exponent_kernel(OzView v, int* E, long estride) {
   __shared__ int sh[8][kT + 1];
   const int tx = threadIdx.x, ty = threadIdx.y;
   const long r0 = (long)blockIdx.y * kT;
   const int batch = blockIdx.z, bh = batch / v.nblo, bl = batch % v.nblo;
-  const long Kt = (long)v.K * v.G;
+  const long Kt = oz_kcount(v, bl), kbase = oz_kbase(v, bl);
   const bool kfast = (v.sK == 1 && v.sR != 1);
   int em[kT / 8];
 #pragma unroll
@@ -440,7 +450,7 @@ __global__ void oz_exponent_kernel(OzView v, int* E) {
       const int i = ty + 8 * j;
       const long r = kfast ? r0 + i : r0 + tx, k = kfast ? k0 + tx : k0 + i;
       if (r < v.rows && k < Kt) {
-        const long long b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, k)]);
+        const long long b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k)]);
         if (b & 0x7FFFFFFFFFFFFFFFll) em[j] = max(em[j], exp_bits(b));
       }
     }
@@ -451,7 +461,7 @@ __global__ void oz_exponent_kernel(OzView v, int* E) {
       int m = em[j];
       for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
       const long r = r0 + ty + 8 * j;
-      if (tx == 0 && r < v.rows && m > kEmptyRow) atomicMax(&E[(long)batch * v.rows + r], m);
+      if (tx == 0 && r < v.rows && m > kEmptyRow) atomicMax(&E[(long)batch * estride + r], m);
     }
     return;
   }
@@ -463,7 +473,7 @@ __global__ void oz_exponent_kernel(OzView v, int* E) {
   if (ty == 0) {
     for (int i = 1; i < 8; ++i) m = max(m, sh[i][tx]);
     const long r = r0 + tx;
-    if (r < v.rows && m > kEmptyRow) atomicMax(&E[(long)batch * v.rows + r], m);
+    if (r < v.rows && m > kEmptyRow) atomicMax(&E[(long)batch * estride + r], m);
   }
 }
 
@@ -472,10 +482,10 @@ __global__ void oz_exponent_kernel(OzView v, int* E) {
 // (the tiled kernel above reads 256 bytes per K index there, which wastes DRAM pages
 // when K is strided). Blocks split K into chunks; loads are unrolled four deep.
 constexpr int kER = 256;
-__global__ void __launch_bounds__(kER) oz_exponent_rows_kernel(OzView v, int* E, long kchunk) {
+__global__ void __launch_bounds__(kER) oz_exponent_rows_kernel(OzView v, int* E, long estride, long kchunk) {
   const long r = (long)blockIdx.y * kER + threadIdx.x;
   const int batch = blockIdx.z, bh = batch / v.nblo, bl = batch % v.nblo;
-  const long Kt = (long)v.K * v.G;
+  const long Kt = oz_kcount(v, bl), kbase = oz_kbase(v, bl);
   const long k0 = (long)blockIdx.x * kchunk, k1 = k0 + kchunk < Kt ? k0 + kchunk : Kt;
   if (r >= v.rows) return;
   int em = kEmptyRow;
@@ -483,16 +493,16 @@ __global__ void __launch_bounds__(kER) oz_exponent_rows_kernel(OzView v, int* E,
   for (; k + 4 <= k1; k += 4) {
     long long b[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) b[u] = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, k + u)]);
+    for (int u = 0; u < 4; ++u) b[u] = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k + u)]);
 #pragma unroll
     for (int u = 0; u < 4; ++u)
       if (b[u] & 0x7FFFFFFFFFFFFFFFll) em = max(em, exp_bits(b[u]));
   }
   for (; k < k1; ++k) {
-    const long long b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, k)]);
+    const long long b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k)]);
     if (b & 0x7FFFFFFFFFFFFFFFll) em = max(em, exp_bits(b));
   }
-  if (em > kEmptyRow) atomicMax(&E[(long)batch * v.rows + r], em);
+  if (em > kEmptyRow) atomicMax(&E[(long)batch * estride + r], em);
 }
 
 // Slice s of 2^-E[row] entry, written tiled: element (batch, row, k) of slice s at
@@ -505,8 +515,8 @@ __global__ void __launch_bounds__(kER) oz_exponent_rows_kernel(OzView v, int* E,
 // operand is read along its unit-stride direction (512 bytes per warp pair) and every
 // output row of every slice is written as one full 128-byte line.
 constexpr int kST = 64;
-__global__ void __launch_bounds__(256) oz_slice_kernel(OzView v, const int* E, __nv_bfloat16* S, long Kpad, int TR,
-                                                       int nrt) {
+__global__ void __launch_bounds__(256) oz_slice_kernel(OzView v, const int* E, long estride, __nv_bfloat16* S,
+                                                       long sbatch, long Kpad, int TR, int nrt) {
   __shared__ long long t[kST][kST + 1];  // [row][k]
   const int tx = threadIdx.x, ty = threadIdx.y;
   const bool kfast = (v.sK == 1 && v.sR != 1);
@@ -514,14 +524,14 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzView v, const int* E, _
   // read neighbouring memory
   const long r0 = (long)(kfast ? blockIdx.y : blockIdx.x) * kST, k0 = (long)(kfast ? blockIdx.x : blockIdx.y) * kST;
   const int batch = blockIdx.z, bh = batch / v.nblo, bl = batch % v.nblo;
-  const long Kt = (long)v.K * v.G;
+  const long Kt = oz_kcount(v, bl), kbase = oz_kbase(v, bl);
   const long nkb = Kpad / 64;
 #pragma unroll 4
   for (int j = 0; j < kST / 4; ++j) {
     const int i = ty + 4 * j;
     const long r = kfast ? r0 + i : r0 + tx, k = kfast ? k0 + tx : k0 + i;
     long long b = 0;
-    if (r < v.rows && k < Kt) b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, k)]);
+    if (r < v.rows && k < Kt) b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k)]);
     if (kfast) t[i][tx] = b;
     else t[tx][i] = b;
   }
@@ -535,7 +545,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzView v, const int* E, _
     const int idx = lin + 256 * rep, i = idx >> 3, kq = (idx & 7) * 8;
     const long r = r0 + i, k = k0 + kq;
     if (r >= (long)nrt * TR || k >= Kpad) continue;
-    const int e = r < v.rows ? E[(long)batch * v.rows + r] : kEmptyRow;
+    const int e = r < v.rows ? E[(long)batch * estride + r] : kEmptyRow;
     uint32_t w[kSlices][4];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
@@ -565,7 +575,7 @@ __global__ void __launch_bounds__(256) oz_slice_kernel(OzView v, const int* E, _
       }
     }
     uint4* out = reinterpret_cast<uint4*>(
-        S + ((((long)batch * nrt + r / TR) * nkb + (k >> 6)) * kSlices * TR + r % TR) * 64 + (k & 63));
+        S + (long)batch * sbatch + ((r / TR * nkb + (k >> 6)) * kSlices * TR + r % TR) * 64 + (k & 63));
 #pragma unroll
     for (int sl = 0; sl < kSlices; ++sl)
       out[(long)sl * sstride / 8] = make_uint4(w[sl][0], w[sl][1], w[sl][2], w[sl][3]);
@@ -587,18 +597,30 @@ void encode_slices(CUtensorMap* map, const __nv_bfloat16* p, int tile_rows, long
 
 }  // namespace
 
+size_t ozaki_slice_bytes(long batches, long rows, long Kpad, int tile_rows) {
+  return sizeof(__nv_bfloat16) * (size_t)(batches * kSlices * ((rows + tile_rows - 1) / tile_rows * tile_rows) * Kpad);
+}
+
 void ozaki_slice(attn_ctx* ctx, const OzView& v, long Kpad, int tile_rows, DevBuf& slices, DevBuf& exps) {
+  const long nb = (long)v.nbhi * v.nblo;
+  slices.reserve(ozaki_slice_bytes(nb, v.rows, Kpad, tile_rows));
+  exps.reserve(sizeof(int) * (size_t)(nb * v.rows));
+  const long nrt = (v.rows + tile_rows - 1) / tile_rows;
+  ozaki_slice_to(ctx, v, Kpad, tile_rows, slices.as<__nv_bfloat16>(), exps.as<int>(),
+                 nrt * tile_rows * Kpad * kSlices, v.rows);
+}
+
+void ozaki_slice_to(attn_ctx* ctx, const OzView& v, long Kpad, int tile_rows, __nv_bfloat16* slices, int* exps,
+                    long slice_stride, long exp_stride) {
   const long nb = (long)v.nbhi * v.nblo;
   ATTN_REQUIRE(nb <= 65535, ATTN_EUNSUPPORTED, "too many operand batches for the split GEMM");
   const int nrt = (v.rows + tile_rows - 1) / tile_rows;
   const long padded = (long)nrt * tile_rows;
   ATTN_REQUIRE(nb * nrt * (Kpad / 64) * kSlices < (1L << 31), ATTN_EUNSUPPORTED, "operand too large for the split GEMM");
-  slices.reserve(sizeof(__nv_bfloat16) * (size_t)(nb * kSlices * padded * Kpad));
-  exps.reserve(sizeof(int) * (size_t)(nb * v.rows));
   cudaStream_t st = ctx->stream;
   const long ne = nb * v.rows;
-  fill_int_kernel<<<(int)std::min<long>((ne + 255) / 256, 4096), 256, 0, st>>>(exps.as<int>(), ne, kEmptyRow);
-  const long Kt = (long)v.K * v.G;
+  fill_int_kernel<<<(int)std::min<long>((ne + 255) / 256, 4096), 256, 0, st>>>(exps, nb, v.rows, exp_stride, kEmptyRow);
+  const long Kt = v.kpart ? v.kpart : (long)v.K * v.G;
   const long rt = (v.rows + kT - 1) / kT;
   ATTN_REQUIRE(rt <= 65535, ATTN_EUNSUPPORTED, "too many rows for the split GEMM");
   dim3 blk(kT, 8);
@@ -608,20 +630,87 @@ void ozaki_slice(attn_ctx* ctx, const OzView& v, long Kpad, int tile_rows, DevBu
     const long nchunk = std::max<long>(1, std::min<long>((Kt + 63) / 64, 2048 / std::max<long>(rb * nb, 1)));
     const long kchunk = (Kt + nchunk - 1) / nchunk;
     dim3 ge((unsigned)((Kt + kchunk - 1) / kchunk), (unsigned)rb, (unsigned)nb);
-    oz_exponent_rows_kernel<<<ge, kER, 0, st>>>(v, exps.as<int>(), kchunk);
+    oz_exponent_rows_kernel<<<ge, kER, 0, st>>>(v, exps, exp_stride, kchunk);
   } else {
     // exponent pass: k tiles folded so that the grid stays modest
     const long kt = (Kt + kT - 1) / kT;
     dim3 ge((unsigned)std::min<long>(kt, std::max<long>(1, 8192 / std::max<long>(rt * nb, 1))), (unsigned)rt,
             (unsigned)nb);
-    oz_exponent_kernel<<<ge, blk, 0, st>>>(v, exps.as<int>());
+    oz_exponent_kernel<<<ge, blk, 0, st>>>(v, exps, exp_stride);
   }
   const bool kfast = (v.sK == 1 && v.sR != 1);
   const unsigned nkt = (unsigned)(Kpad / kST), nrb = (unsigned)((padded + kST - 1) / kST);
   dim3 gs(kfast ? nkt : nrb, kfast ? nrb : nkt, (unsigned)nb);
   ATTN_REQUIRE(gs.y <= 65535, ATTN_EUNSUPPORTED, "operand too large for the split GEMM");
-  oz_slice_kernel<<<gs, dim3(kST, 4), 0, st>>>(v, exps.as<int>(), slices.as<__nv_bfloat16>(), Kpad, tile_rows, nrt);
+  oz_slice_kernel<<<gs, dim3(kST, 4), 0, st>>>(v, exps, exp_stride, slices, slice_stride, Kpad, tile_rows, nrt);
   ctx->launches += 3;
+  ATTN_CHECK_CUDA(cudaGetLastError());
+}
+
+namespace {
+
+constexpr size_t kOzSmem = 1024 + 2 * (size_t)kQBufBytes + (size_t)kPStages * kPBytes + 256;
+
+void oz_prepare(attn_ctx* ctx) {
+  static bool attr = false;
+  if (!attr) {
+    ATTN_CHECK_CUDA(cudaFuncSetAttribute(ozaki_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem));
+    attr = true;
+  }
+  ctx->oz_err.reserve(sizeof(int));
+  if (!ctx->oz_err_init) {
+    ATTN_CHECK_CUDA(cudaMemsetAsync(ctx->oz_err.p, 0, sizeof(int), ctx->stream));
+    ctx->oz_err_init = true;
+  }
+}
+
+// persistent: one CTA per SM (the shared-memory ring allows one), at most one per tile
+void oz_launch(attn_ctx* ctx, const OzMaps& maps, OzParams& prm) {
+  prm.err = ctx->oz_err.as<int>();
+  prm.tiles = (long)((prm.N + kQRows - 1) / kQRows) * ((prm.M + 127) / 128) * prm.Bhi * prm.Blo;
+  const int grid = (int)std::min<long>(prm.tiles, std::max(ctx->num_sms, 1));
+  ozaki_gemm_kernel<<<grid, kOzThreads, kOzSmem, ctx->stream>>>(maps, prm);
+  ctx->launches++;
+}
+
+}  // namespace
+
+int oz_kparts(int M, int N, long K, int sms) {
+  const long tiles = (long)((M + 127) / 128) * ((N + kQRows - 1) / kQRows), nkb = (K + 63) / 64;
+  long best = 0;
+  int at = 1;
+  for (long per = std::min<long>(nkb, 16); per >= std::min<long>(nkb, 4); --per) {
+    // K blocks of the busiest CTA, and two more per tile for its prologue and epilogue
+    const long parts = (nkb + per - 1) / per, cost = (tiles * parts + sms - 1) / sms * (per + 2);
+    if (!best || cost < best) {
+      best = cost;
+      at = (int)per;
+    }
+  }
+  return 64 * at;
+}
+
+void gemm_f64_presliced(attn_ctx* ctx, const __nv_bfloat16* ps, const int* pe, int M, const OzView& q, double* C) {
+  oz_prepare(ctx);
+  const long nkb = q.kpart / 64;
+  const int nrtP = (M + 127) / 128, nrtQ = (q.rows + kQRows - 1) / kQRows;
+  ctx->prof_begin(3);
+  ozaki_slice(ctx, q, q.kpart, kQRows, ctx->oz_ws[2], ctx->oz_ws[3]);
+  OzMaps maps;
+  encode_slices(&maps.p, ps, 128, (long)q.nblo * nrtP * nkb * kSlices);
+  encode_slices(&maps.q, ctx->oz_ws[2].as<__nv_bfloat16>(), kQRows, (long)q.nblo * nrtQ * nkb * kSlices);
+  OzParams prm;
+  prm.M = M; prm.N = q.rows; prm.nkb = (int)nkb;
+  prm.nrtP = nrtP; prm.nrtQ = nrtQ;
+  prm.Bhi = 1; prm.Blo = q.nblo;
+  prm.p_hi = prm.q_hi = 0;
+  prm.p_lo = prm.q_lo = 1;
+  prm.EP = pe;
+  prm.EQ = ctx->oz_ws[3].as<int>();
+  prm.C = C; prm.c_rs = 1; prm.c_cs = M; prm.c_bhi = 0; prm.c_blo = (long)M * q.rows;
+  prm.alpha_rest = 1.0; prm.alpha_exp = 0; prm.beta = 0.0;
+  oz_launch(ctx, maps, prm);
+  ctx->prof_end(3, 2.0 * M * q.rows * (double)q.K * q.G);
   ATTN_CHECK_CUDA(cudaGetLastError());
 }
 
@@ -656,17 +745,7 @@ void gemm_f64_ozaki(attn_ctx* ctx, const GemmF64& g0) {
   // K per launch <= 65536 (int64 headroom): groups of G
   const int gstep = std::max(1, (int)std::min<long>(g0.G, 65536L / std::max(g0.K, 1)));
   ATTN_REQUIRE(g0.K <= 65536, ATTN_EUNSUPPORTED, "K above 65536 for the split GEMM");
-  const size_t smem = 1024 + 2 * (size_t)kQBufBytes + (size_t)kPStages * kPBytes + 256;
-  static bool attr = false;
-  if (!attr) {
-    ATTN_CHECK_CUDA(cudaFuncSetAttribute(ozaki_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
-  ctx->oz_err.reserve(sizeof(int));
-  if (!ctx->oz_err_init) {
-    ATTN_CHECK_CUDA(cudaMemsetAsync(ctx->oz_err.p, 0, sizeof(int), ctx->stream));
-    ctx->oz_err_init = true;
-  }
+  oz_prepare(ctx);
   const double fl = 2.0 * g0.M * g0.N * (double)g0.K * g0.G * g0.Bhi * g0.Blo;
   ctx->prof_begin(3);
   for (int ga = 0; ga < g0.G; ga += gstep) {
@@ -701,12 +780,7 @@ void gemm_f64_ozaki(attn_ctx* ctx, const GemmF64& g0) {
       prm.alpha_rest = pow2 ? (fr < 0 ? -1.0 : 1.0) : g0.alpha;
     }
     prm.beta = ga == 0 ? g0.beta : 1.0;
-    prm.err = ctx->oz_err.as<int>();
-    // persistent: one CTA per SM (the shared-memory ring allows one), at most one per tile
-    prm.tiles = (long)((N + kQRows - 1) / kQRows) * ((M + 127) / 128) * g0.Bhi * g0.Blo;
-    const int grid = (int)std::min<long>(prm.tiles, std::max(ctx->num_sms, 1));
-    ozaki_gemm_kernel<<<grid, kOzThreads, smem, ctx->stream>>>(maps, prm);
-    ctx->launches++;
+    oz_launch(ctx, maps, prm);
   }
   ctx->prof_end(3, fl);
   ATTN_CHECK_CUDA(cudaGetLastError());

@@ -68,3 +68,33 @@ def test_repeated_fp64_applications_match_products(shape, counts, nt):
         assert np.all(np.abs(host(y) - ref) <= 2 * n * 2.0 ** -53 * absref), rep
     attn.attn_heff_destroy(H)
     attn.attn_destroy(ctx)
+
+
+@pytest.mark.parametrize("shape,counts", [((64, 64, 64), (140, 130, 150)), ((48, 56, 72), (120, 0, 110)),
+                                          ((33, 40, 130), (60, 300, 90)), ((16, 24, 20), (12, 12, 14))])
+def test_repeated_split_applications_match_products(shape, counts):
+    """f64_split: every application within the split path's tolerance (1e-12 of the largest
+    entry); zero rows of operators and of x stay exact zeros."""
+    attn, ctx = lib_and_ctx({"f64_split": 1})
+    _, pairs, _ = _problem(shape, counts, 0, sum(shape))
+    hint = [None, random_operators(1, shape[1], 3, 11)[0], None]
+    for k, (p, q) in enumerate(SLOTS):
+        if k in pairs:
+            for t, s in zip(pairs[k], (p, q)):
+                if s == 0:
+                    t[:, 5, :] = 0.0
+    keep = [[None if h is None else dev(h) for h in hint], {k: (dev(a), dev(b)) for k, (a, b) in pairs.items()}]
+    H = attn.attn_heff_create(ctx, shape, *keep)
+    for rep in range(3):
+        x = random_vector(shape, 100 + rep)
+        x[5] = 0.0
+        y = dev(np.full(shape, np.nan))
+        attn.attn_heff_apply(H, dev(x), y, attn.ATTN_F64)
+        attn.attn_sync(ctx)
+        ref = _apply(hint, pairs, None, x)
+        got = host(y)
+        assert np.abs(got - ref).max() <= 1e-12 * np.abs(ref).max(), rep
+        if counts[2] == 0:
+            assert np.all(got[5] == 0.0)
+    attn.attn_heff_destroy(H)
+    attn.attn_destroy(ctx)
