@@ -10,9 +10,12 @@
 // orthogonalised against all other columns (A = Q R still holds because every
 // later column was orthogonalised against the zero column).
 //
-// Storage: At[j][row] = A[row][j] (each column contiguous).
-// Per column: [dots] -> [update + dots] -> [update + norm] -> [finalise]
-// with every block reducing the partials itself (no extra reduce launches).
+// One launch per QR (qr_slab_kernel) while the matrix fits the SMs' shared memory. Larger ones
+// go column by column over At[j][row] = A[row][j] (each column contiguous):
+// [dots] -> [update + dots] -> [update + norm] -> [finalise], every block reducing the
+// partials itself.
+#include <cooperative_groups.h>
+
 #include <algorithm>
 #include <cmath>
 
@@ -232,9 +235,290 @@ __global__ void from_columns_kernel(const double* At, int d0, int d1, int d2, in
   }
 }
 
+// ---- the whole QR in one launch
+//
+// Every CTA keeps its rows of A (all columns) in shared memory from the first column to the
+// last, reading and writing the tensor in place. What bounds a QR of this size is the chain of
+// columns, each of which needs sums over all rows, so the two Gram-Schmidt passes share one
+// reduction per column: the second pass of column j - 1 and the first of column j take their
+// products with the same q_i together (delayed reorthogonalisation: D. Bielich, J. Langou,
+// S. Thomas, K. Swirydowicz, I. Yamazaki, E. Boman, "Low-synch Gram-Schmidt with delayed
+// reorthogonalization for Krylov solvers", Parallel Computing 112 (2022)). With c the second
+// coefficients of w = a_{j-1} - Q s, its norm is |w|^2 - |c|^2, and its product with a_j follows
+// from w . a_j. A column that the first pass cancelled to where |c| is no longer small beside
+// |w| takes its second pass alone and repeats the reduction, so the result is as orthogonal as
+// two full passes make it.
+//
+// Reduction: the CTAs of a cluster add their shares through distributed shared memory, each a
+// slice of the values; several clusters meet through global partials and one grid barrier
+// (cooperative launch; the wait is bounded). All sums run in a fixed order.
+// [64, 64, 64] (4096 x 64): 1600 -> 610 us against four launches per column.
+constexpr int kQrT = 256;    // threads
+constexpr int kQrC = 8;      // CTAs per cluster
+constexpr int kQrMaxK = 256;  // columns
+constexpr long long kQrWait = 4000000000LL;  // cycles that the grid barrier waits at most
+
+struct QrSlab {
+  double* T;
+  long rs_hi, rs_lo, cs;  // element (row, col) at (row / rlo) rs_hi + (row % rlo) rs_lo + col cs
+  int rlo, M, k, rows, ld, nclus;
+  double* R;
+  int* defic;      // [k] rank-deficient columns, [k] = 1 when a wait gave up
+  double* part;    // [2][clusters][2 kQrMaxK]
+  unsigned* bar;   // arrivals, CTAs done
+};
+
+namespace cg = cooperative_groups;
+
+struct QrShared {
+  double loc[2][2 * kQrMaxK];  // this CTA's sums (two, so that one cluster barrier suffices)
+  double tot[2 * kQrMaxK];     // sums over all rows
+  double sum[2 * kQrT];        // partial sums of thread groups
+  double nrm0[kQrMaxK], rprev[kQrMaxK], coef[kQrMaxK];
+  double rho, inv, sy;  // of the column being completed
+  int again, dead;
+};
+
+// tot[0 .. nv) = sum of loc over all CTAs; `step` counts the reductions.
+__device__ void qr_reduce(const QrSlab& q, QrShared& sh, int nv, unsigned step) {
+  cg::cluster_group cl = cg::this_cluster();
+  const int rank = (int)cl.block_rank(), cluster = blockIdx.x / kQrC, t = threadIdx.x, buf = step & 1;
+  cl.sync();
+  if (q.nclus == 1) {
+    for (int v = t; v < nv; v += kQrT) {
+      double s = 0.0;
+#pragma unroll
+      for (int r = 0; r < kQrC; ++r) s += *cl.map_shared_rank(&sh.loc[buf][v], r);
+      sh.tot[v] = s;
+    }
+    __syncthreads();
+    return;
+  }
+  const int v0 = nv * rank / kQrC, n = nv * (rank + 1) / kQrC - v0;  // this CTA's slice
+  double* part = q.part + (long)buf * q.nclus * 2 * kQrMaxK;
+  for (int v = t; v < n; v += kQrT) {
+    double s = 0.0;
+#pragma unroll
+    for (int r = 0; r < kQrC; ++r) s += *cl.map_shared_rank(&sh.loc[buf][v0 + v], r);
+    part[(long)cluster * 2 * kQrMaxK + v0 + v] = s;
+  }
+  __syncthreads();
+  if (t == 0 && !sh.dead) {
+    __threadfence();
+    atomicAdd(q.bar, 1u);
+    const unsigned target = (step + 1) * gridDim.x;
+    const long long t0 = clock64();
+    while (*(volatile unsigned*)q.bar < target) {
+      if (clock64() - t0 > kQrWait) {
+        sh.dead = 1;
+        q.defic[q.k] = 1;
+        break;
+      }
+    }
+    __threadfence();
+  }
+  __syncthreads();
+  // the slice over the clusters, four partial sums per value
+  for (int e = t; e < 4 * n; e += kQrT) {
+    const int v = e >> 2, h = e & 3;
+    double s = 0.0;
+    for (int c = h; c < q.nclus; c += 4) s += __ldcg(part + (long)c * 2 * kQrMaxK + v0 + v);
+    sh.sum[e] = s;
+  }
+  __syncthreads();
+  for (int e = t; e < n * kQrC; e += kQrT) {
+    const int v = e / kQrC, r = e % kQrC;
+    *cl.map_shared_rank(&sh.tot[v0 + v], r) = (sh.sum[4 * v] + sh.sum[4 * v + 1]) + (sh.sum[4 * v + 2] + sh.sum[4 * v + 3]);
+  }
+  cl.sync();
+}
+
+__global__ void __launch_bounds__(kQrT) qr_slab_kernel(const QrSlab q) {
+  extern __shared__ double slab[];  // [rows][ld], ld odd: rows and columns both conflict-free
+  __shared__ QrShared sh;
+  const int t = threadIdx.x, k = q.k, ld = q.ld;
+  const int r0 = blockIdx.x * q.rows, n = max(0, min(q.rows, q.M - r0));
+  auto at = [&](int r, int c) {
+    const int g = r0 + r;
+    return (long)(g / q.rlo) * q.rs_hi + (long)(g % q.rlo) * q.rs_lo + (long)c * q.cs;
+  };
+  if (t == 0) sh.dead = 0;
+  if (t == 0 && blockIdx.x == 0) q.defic[k] = 0;
+  if (q.cs == 1) {
+    for (int e = t; e < n * k; e += kQrT) slab[e / k * ld + e % k] = q.T[at(e / k, e % k)];
+  } else {
+    for (int e = t; e < n * k; e += kQrT) slab[e % n * ld + e / n] = q.T[at(e % n, e / n)];
+  }
+  __syncthreads();
+
+  // loc = sums over this CTA's rows of columns 0 .. nc - 1 with column x (and, if y >= 0, y; with
+  // themselves if x < 0): threads take a column and every G-th row
+  auto dots = [&](int nc, int x, int y, double* loc) {
+    int W = 16;
+    while (W < nc) W *= 2;
+    const int G = kQrT / W, i = t % W, g = t / W;
+    double a0 = 0.0, a1 = 0.0, b0 = 0.0, b1 = 0.0;
+    if (i < nc) {
+      int r = g;
+      for (; r + G < n; r += 2 * G) {
+        const double *p = slab + r * ld, *p2 = p + G * ld;
+        const double v = p[i], v2 = p2[i];
+        a0 = fma(v, x < 0 ? v : p[x], a0);
+        a1 = fma(v2, x < 0 ? v2 : p2[x], a1);
+        if (y >= 0) {
+          b0 = fma(v, p[y], b0);
+          b1 = fma(v2, p2[y], b1);
+        }
+      }
+      if (r < n) {
+        const double* p = slab + r * ld;
+        a0 = fma(p[i], x < 0 ? p[i] : p[x], a0);
+        if (y >= 0) b0 = fma(p[i], p[y], b0);
+      }
+    }
+    sh.sum[t] = a0 + a1;
+    sh.sum[kQrT + t] = b0 + b1;
+    __syncthreads();
+    for (int v = t; v < (y >= 0 ? 2 * nc : nc); v += kQrT) {
+      const double* p = sh.sum + (v >= nc ? kQrT + v - nc : v);
+      double s = p[0];
+      for (int h = 1; h < G; ++h) s += p[h * W];
+      loc[v] = s;
+    }
+    __syncthreads();
+  };
+  // column x -= sum_{i < nc} Q_i cx_i, scaled by f; column y (if >= 0) -= sum Q_i cy_i + sy times the
+  // new column x: threads take a row and every P-th column
+  auto update = [&](int nc, int x, const double* cx, double f, int y, const double* cy, double sy) {
+    int W = 16;
+    while (W < n) W *= 2;
+    const int P = kQrT / W, r = t % W, p = t / W;
+    double a0 = 0.0, b0 = 0.0, a1 = 0.0, b1 = 0.0;
+    if (r < n) {
+      const double* row = slab + r * ld;
+      int i = p;
+      for (; i + P < nc; i += 2 * P) {
+        const double v = row[i], v2 = row[i + P];
+        a0 = fma(v, cx[i], a0);
+        a1 = fma(v2, cx[i + P], a1);
+        if (y >= 0) {
+          b0 = fma(v, cy[i], b0);
+          b1 = fma(v2, cy[i + P], b1);
+        }
+      }
+      if (i < nc) {
+        a0 = fma(row[i], cx[i], a0);
+        if (y >= 0) b0 = fma(row[i], cy[i], b0);
+      }
+    }
+    sh.sum[t] = a0 + a1;
+    sh.sum[kQrT + t] = b0 + b1;
+    __syncthreads();
+    if (t < n) {
+      double a = sh.sum[t], b = sh.sum[kQrT + t];
+      for (int h = 1; h < P; ++h) {
+        a += sh.sum[h * W + t];
+        b += sh.sum[kQrT + h * W + t];
+      }
+      double* row = slab + t * ld;
+      const double u = (row[x] - a) * f;
+      row[x] = u;
+      if (y >= 0) row[y] = fma(-sy, u, row[y] - b);
+    }
+    __syncthreads();
+  };
+
+  unsigned step = 0;
+  dots(k, -1, -1, sh.loc[0]);
+  qr_reduce(q, sh, k, step++);
+  for (int i = t; i < k; i += kQrT) {
+    sh.nrm0[i] = sqrt(sh.tot[i]);
+    sh.rprev[i] = 0.0;
+  }
+  __syncthreads();
+  for (int j = 1; j <= k; ++j) {  // column w = j - 1 is completed, column j takes its first pass
+    const int w = j - 1, y = j < k ? j : -1;
+    for (int again = 0;; ++again) {
+      dots(j, w, y, sh.loc[step & 1]);
+      qr_reduce(q, sh, y >= 0 ? 2 * j : j, step++);
+      // tot: c_i (i < w), |w|^2; s_i, w . a_j. Every CTA has the same sums and takes the same
+      // way; one warp works the scalars out (an FP64 instruction costs a warp 16 cycles of the SM)
+      if (t < 32) {
+        const double w2 = sh.tot[w];
+        const float sc = rsqrtf((float)w2);
+        float fc = 0.0f;  // |c|^2 / |w|^2
+        for (int i = t; i < w; i += 32) {
+          const double c = sh.tot[i];
+          const float f = (float)c * sc;
+          fc = fmaf(f, f, fc);
+          sh.rprev[i] += c;
+        }
+        for (int o = 16; o > 0; o >>= 1) fc += __shfl_xor_sync(0xffffffffu, fc, o);
+        // c below 1e-9 of w, the usual case: its square is nothing beside |w|^2, and FP32 is enough
+        // for c . s, a correction of that size
+        double cc = 0.0, cs = 0.0;
+        if (fc <= 1e-18f) {
+          float fs = 0.0f;
+          for (int i = t; i < w && y >= 0; i += 32) fs = fmaf((float)sh.tot[i], (float)sh.tot[j + i], fs);
+          for (int o = 16; o > 0; o >>= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);
+          cs = (double)fs;
+        } else {
+          for (int i = t; i < w; i += 32) {
+            const double c = sh.tot[i];
+            cc = fma(c, c, cc);
+            if (y >= 0) cs = fma(c, sh.tot[j + i], cs);
+          }
+          for (int o = 16; o > 0; o >>= 1) {
+            cc += __shfl_xor_sync(0xffffffffu, cc, o);
+            cs += __shfl_xor_sync(0xffffffffu, cs, o);
+          }
+        }
+        if (t == 0) {
+          const double d = w2 - cc, n0 = sh.nrm0[w];
+          const double inv = rsqrt(d), rho = d > 0.0 ? d * inv : (d == d ? 0.0 : d);  // (a NaN stays one)
+          const bool ok = rho > 1e-13 * n0 && rho > 1e-300;
+          sh.again = cc > 0.25 * w2 && again < 3 && w2 > 1e-26 * n0 * n0;
+          sh.rho = ok ? rho : 0.0;
+          sh.inv = ok ? inv : 0.0;
+          sh.sy = ok && y >= 0 ? (sh.tot[j + w] - cs) * inv : 0.0;
+        }
+      }
+      __syncthreads();
+      if (!sh.again) break;
+      update(w, w, sh.tot, 1.0, -1, nullptr, 0.0);
+    }
+    const double rho = sh.rho, inv = sh.inv, sy = sh.sy;
+    const bool ok = rho > 0.0;
+    if (blockIdx.x == 0) {
+      for (int i = t; i < k; i += kQrT)
+        q.R[(long)i * k + w] = i < w ? sh.rprev[i] : (i == w ? rho : 0.0);
+      if (t == 0) q.defic[w] = ok ? 0 : 1;
+    }
+    update(w, w, sh.tot, inv, y, sh.tot + j, sy);
+    if (y >= 0)
+      for (int i = t; i <= w; i += kQrT) sh.rprev[i] = i < w ? sh.tot[j + i] : sy;
+    __syncthreads();
+  }
+  if (q.cs == 1) {
+    for (int e = t; e < n * k; e += kQrT) q.T[at(e / k, e % k)] = slab[e / k * ld + e % k];
+  } else {
+    for (int e = t; e < n * k; e += kQrT) q.T[at(e % n, e / n)] = slab[e % n * ld + e / n];
+  }
+  if (t == 0 && q.nclus > 1) {  // the last CTA leaves the barrier as it found it
+    __threadfence();
+    if (atomicAdd(q.bar + 1, 1u) == gridDim.x - 1) {
+      q.bar[0] = 0;
+      q.bar[1] = 0;
+    }
+  }
+  cg::this_cluster().sync();  // no CTA leaves while another may read its shared memory
+}
+
 int grid1(long n) { return (int)std::max<long>(1, std::min<long>((n + 255) / 256, 4096)); }
 
 }  // namespace
+
+static void qr_complete(attn_ctx* ctx, double* At, long M, int k, const std::vector<int>& hdef, double* part);
 
 void qr_columns(attn_ctx* ctx, double* At, long M, int k, double* R, QRWork& w) {
   ATTN_REQUIRE(k >= 1 && M >= k, ATTN_EINVAL, "QR needs M >= k >= 1 (link wider than its other side)");
@@ -270,6 +554,13 @@ void qr_columns(attn_ctx* ctx, double* At, long M, int k, double* R, QRWork& w) 
   std::vector<int> hdef(k);
   ATTN_CHECK_CUDA(cudaMemcpyAsync(hdef.data(), def, sizeof(int) * k, cudaMemcpyDeviceToHost, s));
   ATTN_CHECK_CUDA(cudaStreamSynchronize(s));
+  qr_complete(ctx, At, M, k, hdef, part);
+}
+
+// Replaces the rank-deficient columns of At by unit vectors orthogonalised against the others.
+static void qr_complete(attn_ctx* ctx, double* At, long M, int k, const std::vector<int>& hdef, double* part) {
+  cudaStream_t s = ctx->stream;
+  const size_t hsh = sizeof(double) * k;
   for (int j = 0; j < k; ++j) {
     if (!hdef[j]) continue;
     bool ok = false;
@@ -284,6 +575,104 @@ void qr_columns(attn_ctx* ctx, double* At, long M, int k, double* R, QRWork& w) 
       ok = nrm > 0.5;
     }
     ATTN_REQUIRE(ok, ATTN_ENOTISOMETRIC, "QR could not complete a rank-deficient column");
+  }
+}
+
+void qr_tensor(attn_ctx* ctx, double* T, const int d[3], int slot, double* R, QRWork& w) {
+  const long V = (long)d[0] * d[1] * d[2];
+  const int k = d[slot];
+  const long M = V / std::max(k, 1);
+  ATTN_REQUIRE(k >= 1 && M >= k, ATTN_EINVAL, "QR needs M >= k >= 1 (link wider than its other side)");
+  QrSlab q;
+  q.ld = k | 1;
+  constexpr size_t kSmemMax = 200 * 1024;
+  static int most = 0;  // clusters that are resident together with a full slab per SM
+  if (!most) {
+    ATTN_CHECK_CUDA(cudaFuncSetAttribute(qr_slab_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(kQrC);
+    c.blockDim = dim3(kQrT);
+    c.dynamicSmemBytes = kSmemMax;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeClusterDimension;
+    attr.val.clusterDim.x = kQrC;
+    attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+    c.attrs = &attr;
+    c.numAttrs = 1;
+    int nc = 0;
+    ATTN_CHECK_CUDA(cudaOccupancyMaxActiveClusters(&nc, qr_slab_kernel, &c));
+    most = std::max(nc, 1);
+  }
+  // Clusters by the cycles of a column: rows x k FP64 FMAs at two per cycle on the busiest SM
+  // (both passes, both products), the cluster barriers and, with more than one cluster, the grid
+  // barrier and the sums over the clusters (measured around 3 us).
+  double best = 0.0;
+  int nclus = 0;
+  for (int c = 1; c <= most; ++c) {
+    const long rows = (M + (long)c * kQrC - 1) / ((long)c * kQrC);
+    if (rows > kQrT || sizeof(double) * rows * q.ld > kSmemMax || k > kQrMaxK) continue;
+    const double cost = (double)rows * k + 1500.0 + (c > 1 ? 6000.0 + 20.0 * c : 0.0);
+    if (!nclus || cost < best) {
+      best = cost;
+      nclus = c;
+    }
+  }
+  if (!nclus) {
+    w.cols.reserve(sizeof(double) * V);
+    tensor_to_columns(ctx, T, d, slot, w.cols.as<double>());
+    qr_columns(ctx, w.cols.as<double>(), M, k, R, w);
+    columns_to_tensor(ctx, w.cols.as<double>(), d, slot, T);
+    return;
+  }
+  q.T = T;
+  q.M = (int)M;
+  q.k = k;
+  q.nclus = nclus;
+  q.rows = (int)((M + (long)nclus * kQrC - 1) / ((long)nclus * kQrC));
+  const long d1 = d[1], d2 = d[2];
+  if (slot == 0) { q.rlo = d[2]; q.rs_hi = d2; q.rs_lo = 1; q.cs = d1 * d2; }
+  else if (slot == 1) { q.rlo = d[2]; q.rs_hi = d1 * d2; q.rs_lo = 1; q.cs = d2; }
+  else { q.rlo = d[1]; q.rs_hi = d1 * d2; q.rs_lo = d2; q.cs = 1; }
+  q.R = R;
+  w.defic.reserve(sizeof(int) * (kQrMaxK + 1));
+  w.part.reserve(sizeof(double) * ((size_t)2 * most * 2 * kQrMaxK + 16));
+  if (!w.bar_init) {
+    w.bar.reserve(2 * sizeof(unsigned));
+    ATTN_CHECK_CUDA(cudaMemsetAsync(w.bar.p, 0, 2 * sizeof(unsigned), ctx->stream));
+    w.bar_init = true;
+  }
+  q.defic = w.defic.as<int>();
+  q.part = w.part.as<double>();
+  q.bar = w.bar.as<unsigned>();
+  cudaLaunchConfig_t c = {};
+  c.gridDim = dim3((unsigned)(nclus * kQrC));
+  c.blockDim = dim3(kQrT);
+  c.dynamicSmemBytes = sizeof(double) * (size_t)q.rows * q.ld;
+  c.stream = ctx->stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeClusterDimension;
+  attr[0].val.clusterDim.x = kQrC;
+  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeCooperative;
+  attr[1].val.cooperative = 1;
+  c.attrs = attr;
+  c.numAttrs = nclus > 1 ? 2 : 1;
+  ATTN_CHECK_CUDA(cudaLaunchKernelEx(&c, qr_slab_kernel, q));
+  ctx->launches++;
+  // rank-deficient columns (rare) and a wait that gave up: host check, one small sync
+  std::vector<int> hdef(k + 1);
+  ATTN_CHECK_CUDA(cudaMemcpyAsync(hdef.data(), q.defic, sizeof(int) * (k + 1), cudaMemcpyDeviceToHost, ctx->stream));
+  ATTN_CHECK_CUDA(cudaStreamSynchronize(ctx->stream));
+  if (hdef[k]) {
+    w.bar_init = false;
+    throw Error{ATTN_ETIMEOUT, "a bounded wait in the QR kernel gave up"};
+  }
+  hdef.pop_back();
+  if (std::any_of(hdef.begin(), hdef.end(), [](int v) { return v != 0; })) {
+    w.cols.reserve(sizeof(double) * V);
+    tensor_to_columns(ctx, T, d, slot, w.cols.as<double>());
+    qr_complete(ctx, w.cols.as<double>(), M, k, hdef, w.part.as<double>());
+    columns_to_tensor(ctx, w.cols.as<double>(), d, slot, T);
   }
 }
 

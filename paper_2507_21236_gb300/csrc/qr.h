@@ -7,7 +7,14 @@ namespace attn {
 
 struct QRWork {
   DevBuf part, part2, nrm0, defic;
+  DevBuf cols;          // column-stored copy of a matrix too large for one launch
+  DevBuf bar;           // grid barrier of the one-launch QR
+  bool bar_init = false;
 };
+
+// In-place QR of T viewed as the matrix with the `slot` index as column: T's entries become Q's,
+// R as below.
+void qr_tensor(attn_ctx* ctx, double* T, const int d[3], int slot, double* R, QRWork& w);
 
 // In-place QR of the column-stored matrix At[k][M] (column j contiguous):
 // on return At holds Q's columns and R (k x k, row-major, device) the

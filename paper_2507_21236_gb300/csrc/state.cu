@@ -101,12 +101,8 @@ void attn_state::init_from_raw(const double* const* raw) {
       normalise_dev(ctx, tensor(n), tensor(n), vol(n), ctx->scal.as<double>());
       continue;
     }
-    const long M = (long)d[0] * d[1];
-    colbuf.reserve(sizeof(double) * vol(n));
     rbuf.reserve(sizeof(double) * d[2] * d[2]);
-    tensor_to_columns(ctx, tensor(n), d, 2, colbuf.as<double>());
-    qr_columns(ctx, colbuf.as<double>(), M, d[2], rbuf.as<double>(), qrw);
-    columns_to_tensor(ctx, colbuf.as<double>(), d, 2, tensor(n));
+    qr_tensor(ctx, tensor(n), d, 2, rbuf.as<double>(), qrw);
   }
   centre = tree.top0();
   env.clear();
@@ -144,12 +140,8 @@ void attn_state::move_centre(int target) {
     const int da[3] = {dim(a, 0), dim(a, 1), dim(a, 2)};
     const int db[3] = {dim(b, 0), dim(b, 1), dim(b, 2)};
     const int k = da[s];
-    const long M = vol(a) / k;
-    colbuf.reserve(sizeof(double) * vol(a));
     rbuf.reserve(sizeof(double) * k * k);
-    tensor_to_columns(ctx, tensor(a), da, s, colbuf.as<double>());
-    qr_columns(ctx, colbuf.as<double>(), M, k, rbuf.as<double>(), qrw);
-    columns_to_tensor(ctx, colbuf.as<double>(), da, s, tensor(a));
+    qr_tensor(ctx, tensor(a), da, s, rbuf.as<double>(), qrw);
     tmpT.reserve(sizeof(double) * vol(b));
     mode_product_f64(ctx, db, back, rbuf.as<double>(), 1, tensor(b), 0, tmpT.as<double>(), 0.0);
     std::swap(T[b], tmpT);
