@@ -182,10 +182,39 @@ inline int grid_for(size_t n, int threads = 256, int cap = 4096) {
 
 }  // namespace
 
-// Launch with the tile shape that wastes least of M and N (grid.y > 65535 is rejected).
+static int sm_count() {
+  static int sms = 0;
+  int dev = 0, n = 0;
+  if (!sms && cudaGetDevice(&dev) == cudaSuccess &&
+      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
+    sms = n;
+  return std::max(sms, 1);
+}
+
+// Tile of g: the one whose busiest SM computes the fewest outputs (FP64 FMAs at two per cycle
+// and SM bound the kernel). A batch too short for a tile per SM takes smaller ones:
+// the 64 x 4096 x 64 product of a centre move 69 -> 37 us with 64 x 32 tiles (128 instead of 64).
+// 5 % for the loads of a 32-wide side.
+static void tile_of(const GemmF64& g, int* bm, int* bn) {
+  const long nb = (long)g.Bhi * g.Blo * g.gsplit, sms = sm_count();
+  double best = 0.0;
+  for (int m : {64, 32})
+    for (int n : {64, 32}) {
+      const long tiles = (long)((g.M + m - 1) / m) * ((g.N + n - 1) / n) * nb;
+      const double cost = (double)((tiles + sms - 1) / sms) * m * n * (m == 32 ? 1.05 : 1.0) * (n == 32 ? 1.05 : 1.0);
+      if (best == 0.0 || cost < best) {
+        best = cost;
+        *bm = m;
+        *bn = n;
+      }
+    }
+}
+
+// (grid.y > 65535 is rejected)
 cudaError_t launch_gemm(cudaStream_t stream, const GemmF64& g) {
-  const bool sm = g.M <= 32, sn = g.N <= 32;
-  const int bm = sm ? 32 : 64, bn = sn ? 32 : 64;
+  int bm, bn;
+  tile_of(g, &bm, &bn);
+  const bool sm = bm == 32, sn = bn == 32;
   dim3 grid((g.N + bn - 1) / bn, (g.M + bm - 1) / bm, (unsigned)std::min<long>((long)g.Bhi * g.Blo * g.gsplit, 65535));
   if (grid.y > 65535) return cudaErrorInvalidValue;
   if (sm && sn) gemm_f64_kernel<32, 32><<<grid, NT, 0, stream>>>(g);
