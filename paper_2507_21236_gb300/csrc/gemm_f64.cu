@@ -240,26 +240,39 @@ static int resident_ctas(const GemmF64& g) {
   return occ[v];
 }
 
-void gemm_f64(attn_ctx* ctx, const GemmF64& g) {
-  if (g.M <= 0 || g.N <= 0 || g.Bhi <= 0 || g.Blo <= 0) return;
-  ATTN_REQUIRE((g.M + 31) / 32 <= 65535, ATTN_EUNSUPPORTED, "GEMM M too large");
-  const double fl = 2.0 * g.M * g.N * (double)g.K * g.G * g.Bhi * g.Blo;
+void gemm_f64(attn_ctx* ctx, const GemmF64& g0) {
+  if (g0.M <= 0 || g0.N <= 0 || g0.Bhi <= 0 || g0.Blo <= 0) return;
+  ATTN_REQUIRE((g0.M + 31) / 32 <= 65535, ATTN_EUNSUPPORTED, "GEMM M too large");
+  const double fl = 2.0 * g0.M * g0.N * (double)g0.K * g0.G * g0.Bhi * g0.Blo;
   // marked contractions of at least ~1e8 FLOP run as exact BF16 slice products when
   // enabled: GB300's FP64 FMA rate is a small fraction of its tensor-core rate. The
   // slicing grid takes at most 65535 distinct batch entries per operand.
-  const long nbA = (g.aBhi ? (long)g.Bhi : 1L) * (g.aBlo ? (long)g.Blo : 1L);
-  const long nbB = (g.bBhi ? (long)g.Bhi : 1L) * (g.bBlo ? (long)g.Blo : 1L);
-  if (ctx->cfg.f64_split && g.split_ok && fl >= 1e8 && std::max(g.M, g.N) >= 32 && nbA <= 65535 &&
+  const long nbA = (g0.aBhi ? (long)g0.Bhi : 1L) * (g0.aBlo ? (long)g0.Blo : 1L);
+  const long nbB = (g0.bBhi ? (long)g0.Bhi : 1L) * (g0.bBlo ? (long)g0.Blo : 1L);
+  if (ctx->cfg.f64_split && g0.split_ok && fl >= 1e8 && std::max(g0.M, g0.N) >= 32 && nbA <= 65535 &&
       nbB <= 65535) {
-    gemm_f64_ozaki(ctx, g);
+    gemm_f64_ozaki(ctx, g0);
     return;
   }
-  const int bm = g.M <= 32 ? 32 : 64, bn = g.N <= 32 ? 32 : 64;
-  const long nb = (long)g.Bhi * g.Blo;
-  const long tiles = (long)((g.N + bn - 1) / bn) * ((g.M + bm - 1) / bm) * nb;
-  const long slots = (long)std::max(ctx->num_sms, 1) * resident_ctas(g);
+  const int bm = g0.M <= 32 ? 32 : 64, bn = g0.N <= 32 ? 32 : 64;
+  const long nb = (long)g0.Bhi * g0.Blo;
+  const long tiles = (long)((g0.N + bn - 1) / bn) * ((g0.M + bm - 1) / bm) * nb;
+  const long slots = (long)std::max(ctx->num_sms, 1) * resident_ctas(g0);
   // split the G reduction when the output tiles fill less than half a wave: as many
-  // groups as keep the whole grid within one wave of resident CTAs
+  // groups as keep the whole grid within one wave of resident CTAs. A reduction over K alone is
+  // first cut into equal pieces of at least 32, from K = 256 on (the renormalised internal operator of a link is
+  // one 64 x 64 product over K = 4096: 4.0 ms on the one SM that had it, 0.06 ms over all)
+  GemmF64 g = g0;
+  if (g.G == 1 && 2 * tiles <= slots && g.K >= 256) {
+    for (int n = (int)std::min<long>(g.K / 32, slots / tiles); n > 1; --n)
+      if (g.K % n == 0) {
+        g.G = n;
+        g.K /= n;
+        g.aG = g.K * g.aK;
+        g.bG = g.K * g.bK;
+        break;
+      }
+  }
   const int ks = (g.G >= 2 && 2 * tiles <= slots) ? (int)std::min<long>(g.G, slots / tiles) : 1;
   ctx->prof_begin(1);
   if (ks > 1) {
