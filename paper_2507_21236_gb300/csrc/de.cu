@@ -520,6 +520,14 @@ void attn_state::probe_expectations(const std::vector<ProbeFactor>& F, const std
     const double* Ax = Px.ops.as<double>();
     const double* By = Py.ops.as<double>();
     double* out = o.ops.as<double>();
+    if (renorm_small_fits(d, xs[0], xs[1], t) && std::max(Px.keys.size(), Py.keys.size()) < 32768) {
+      std::vector<std::pair<int, int>> open;
+      for (size_t r = 0; r < bx.size(); ++r) open.push_back({bx[r], by[r]});
+      for (int i : xi) open.push_back({i, -1});
+      for (int i : yi) open.push_back({-1, i});
+      renorm_small(ctx, Tc, d, t, xs[0], xs[1], Ax, By, nullptr, nullptr, open, out, {}, nullptr, rs_part);
+      continue;
+    }
     if (!gb.empty()) renorm_batch(Tc, d, t, xs[0], xs[1], Ax, bx, By, by, out);
     if (!gx.empty()) renorm_batch(Tc, d, t, xs[0], xs[1], Ax, xi, nullptr, {}, out + (long)gb.size() * osz);
     if (!gy.empty())

@@ -267,6 +267,20 @@ void attn_state::renormalise_into(int n, int slot) {
   const long osz = (long)dt * dt;
   if (!out.open.empty()) out.ops.reserve(sizeof(double) * out.open.size() * osz);
 
+  out.has_hint = Ex.has_hint || Ey.has_hint || !closed.empty();
+  out.hint.reserve(sizeof(double) * osz);
+  if (renorm_small_fits(d, x, y, t) && std::max(Ex.open.size(), Ey.open.size()) < 32768) {
+    std::vector<std::pair<int, int>> open, in;
+    for (size_t r = 0; r < bx.size(); ++r) open.push_back({bx[r], by[r]});
+    for (int i : xi) open.push_back({i, -1});
+    for (int i : yi) open.push_back({-1, i});
+    if (Ex.has_hint) in.push_back({-2, -1});
+    if (Ey.has_hint) in.push_back({-1, -2});
+    for (size_t r = 0; r < cx.size(); ++r) in.push_back({cx[r], cy[r]});
+    renorm_small(ctx, Tc, d, t, x, y, Ex.ops.as<double>(), Ey.ops.as<double>(), Ex.hint.as<double>(),
+                 Ey.hint.as<double>(), open, out.ops.as<double>(), in, out.hint.as<double>(), rs_part);
+    return;
+  }
   const long budget = 1L << 26;  // doubles per intermediate
   const int chunk = (int)std::max<long>(1, std::min<long>(1024, budget / std::max<long>(V, 1)));
   renorm_batch(Tc, d, t, x, y, Ex.ops.as<double>(), bx, Ey.ops.as<double>(), by, out.ops.as<double>());
@@ -275,8 +289,6 @@ void attn_state::renormalise_into(int n, int slot) {
                out.ops.as<double>() + (long)(both.size() + xonly.size()) * osz);
 
   // internal operator: T^T (H_x (x) 1 + 1 (x) H_y + sum_closed A (x) B) T
-  out.has_hint = Ex.has_hint || Ey.has_hint || !closed.empty();
-  out.hint.reserve(sizeof(double) * osz);
   if (!out.has_hint) return;
   rw1.reserve(sizeof(double) * V);
   double* Wsum = rw1.as<double>();

@@ -50,6 +50,15 @@ struct DESetup {
   std::vector<double> lambda;        // [pos] summed spectral-norm shifts
 };
 
+// All products of a link renormalised in one launch, for small tensors (renorm_small.cu):
+// out[r] = T^T (A[open[r].first] on slot x (x) B[open[r].second] on slot y) T over slots x, y with
+// open slot t, and hint = the same summed over `closed` (untouched when that is empty). A product's
+// index -1 stands for the identity, -2 for the slot's internal operator ha / hb.
+bool renorm_small_fits(const int d[3], int x, int y, int t);
+void renorm_small(attn_ctx* ctx, const double* T, const int d[3], int t, int x, int y, const double* A, const double* B,
+                  const double* ha, const double* hb, const std::vector<std::pair<int, int>>& open, double* out,
+                  const std::vector<std::pair<int, int>>& closed, double* hint, DevBuf& part);
+
 }  // namespace attn
 
 struct attn_state {
@@ -77,6 +86,7 @@ struct attn_state {
   attn::QRWork qrw;
   attn::LanczosWork lw, lw2;
   attn::RefineWork rfw;
+  attn::DevBuf rs_part;  // groups of an internal operator (renorm_small)
   attn::DevBuf colbuf, rbuf, tmpT, idxbuf, opsA, opsB, rw1, rw2;
   // The H_eff of the last local step, kept with its device buffers so that the next
   // build reuses them (its operator stacks and their tensor-core copies take hundreds
