@@ -22,8 +22,8 @@
 // factors from their sites to the isometry centre along the tree (the path
 // contraction of Sec. 4.2.1 for all disentanglers at once, with identical
 // partial products shared), then contracting with the centre tensor. The
-// 4x4 iterations of all disentanglers run in one kernel, one thread each,
-// with a one-sided Jacobi SVD.
+// 4x4 iterations of all disentanglers run in one kernel, one warp each (one thread each for
+// de_method 1), with a one-sided Jacobi SVD.
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -181,26 +181,174 @@ __device__ void mera_solve(const double* G, double* u) {
     }
 }
 
-__global__ void de_mera_kernel(DEArgs a) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  if (k >= a.n_de) return;
-  const int b0 = a.ent_begin[k], b1 = a.ent_begin[k + 1];
-  double u[16], g[16], un[16];
-  for (int i = 0; i < 16; ++i) u[i] = a.u_in[16L * k + i];
-  double e = de_energy(a, b0, b1, u);
-  a.e_out[2 * k] = e;
+// The MERA-like update, one warp per disentangler: lanes are the 16 entries of a 4 x 4 matrix,
+// twice (half h of the warp takes every other entry of the environment). An FP64 instruction
+// occupies a warp's scheduler for 64 cycles however many of its lanes work, so a thread
+// doing its matrix products alone costs the same time per multiply-add as 32 of them do here.
+// 16 disentanglers, 20 steps: 4.0 -> 0.41 ms.
+struct DeShared {
+  double u[16], w[2][16], g[16];
+  double M[kMaxEnt][16], C[kMaxEnt][16];
+  double B[16], J[16], rho[16];
+};
+
+__device__ __forceinline__ double warp_add(double v) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// sum_q Tr(M_q u^T C_q u) with u in sh.u
+__device__ double de_energy_warp(DeShared& sh, int n) {
+  const int lane = threadIdx.x & 31, h = lane >> 4, i = (lane >> 2) & 3, j = lane & 3;
+  double e = 0.0;
+  for (int q0 = 0; q0 < n; q0 += 2) {
+    const int q = q0 + h;
+    double w = 0.0, uc = 0.0;
+    if (q < n)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w = fma(sh.C[q][i * 4 + k], sh.u[k * 4 + j], w);
+    __syncwarp();
+    sh.w[h][i * 4 + j] = w;
+    __syncwarp();
+    if (q < n) {
+#pragma unroll
+      for (int k = 0; k < 4; ++k) uc = fma(sh.u[k * 4 + i], sh.w[h][k * 4 + j], uc);
+      e = fma(sh.M[q][j * 4 + i], uc, e);
+    }
+  }
+  return warp_add(e);
+}
+
+// Gamma (de_gamma) of u in sh.u, into sh.g
+__device__ void de_gamma_warp(DeShared& sh, int n, double lambda) {
+  const int lane = threadIdx.x & 31, h = lane >> 4, i = (lane >> 2) & 3, j = lane & 3;
+  double g = 0.0;
+  for (int q0 = 0; q0 < n; q0 += 2) {
+    const int q = q0 + h;
+    double w = 0.0;
+    if (q < n)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) w = fma(sh.u[k * 4 + i], sh.C[q][k * 4 + j], w);
+    __syncwarp();
+    sh.w[h][i * 4 + j] = w;
+    __syncwarp();
+    if (q < n)
+#pragma unroll
+      for (int k = 0; k < 4; ++k) g = fma(sh.M[q][i * 4 + k], sh.w[h][k * 4 + j], g);
+  }
+  g += __shfl_xor_sync(0xffffffffu, g, 16);
+  double r = 0.0;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) r = fma(sh.rho[i * 4 + k], sh.u[j * 4 + k], r);
+  g = fma(-lambda, r, g);
+  __syncwarp();
+  if (h == 0) sh.g[i * 4 + j] = g;
+  __syncwarp();
+}
+
+// u = -V W^T for G = W diag(s) V^T (G in sh.g, u into sh.u): one-sided Jacobi on the columns of
+// G, two rotations at a time. Lane (m, r, c) holds entry (r, c) of B (m = 0) or of the
+// accumulated rotations J (m = 1). The angle comes from FP32 (any angle that reduces the
+// product of the columns will do, and the last sweeps take it to rounding), its cosine and sine
+// from FP64, so the rotations stay orthogonal.
+__device__ void mera_solve_warp(DeShared& sh) {
+  const int lane = threadIdx.x & 31, r = (lane >> 2) & 3, c = lane & 3;
+  double v = lane < 16 ? sh.g[lane] : (r == c ? 1.0 : 0.0);
+  for (int sweep = 0; sweep < 60; ++sweep) {
+    bool more = false;
+#pragma unroll
+    for (int round = 1; round < 4; ++round) {  // pairs of columns c, c ^ round
+      const double w = __shfl_xor_sync(0xffffffffu, v, round);
+      double nn = v * v, x = v * w;
+      nn += __shfl_xor_sync(0xffffffffu, nn, 4);
+      x += __shfl_xor_sync(0xffffffffu, x, 4);
+      nn += __shfl_xor_sync(0xffffffffu, nn, 8);
+      x += __shfl_xor_sync(0xffffffffu, x, 8);
+      nn = __shfl_sync(0xffffffffu, nn, lane & 15);
+      x = __shfl_sync(0xffffffffu, x, lane & 15);
+      const double mm = __shfl_xor_sync(0xffffffffu, nn, round);
+      const bool low = c < (c ^ round);  // this lane's column is the pair's first
+      const double a = low ? nn : mm, b = low ? mm : nn;
+      const int ea = (__double2hiint(a) >> 20) & 0x7FF, eb = (__double2hiint(b) >> 20) & 0x7FF;
+      // (entries below 2^-1000 of a double's range, or NaN: nothing to rotate)
+      bool rot = x != 0.0 && a > 0.0 && b > 0.0 && ea > 0 && eb > 0;
+      double cs = 1.0, sn = 0.0;
+      if (rot) {
+        // common power of two out, so that FP32 holds the three sums
+        const int ex = max(ea, eb);
+        const double sc = __hiloint2double((2046 - ex) << 20, 0);
+        const float fa = (float)(a * sc), fb = (float)(b * sc), fx = (float)(x * sc);
+        // |x| / sqrt(a b) > 1e-16, in two factors that FP32 holds
+        const float ratio = fabsf(fx) * rsqrtf(fmaxf(fa, fb));
+        rot = ratio > 1e-16f * sqrtf(fminf(fa, fb));
+        more = more || ratio > 1e-15f * sqrtf(fminf(fa, fb));
+        if (rot && fx != 0.0f) {
+          const float zeta = (fb - fa) / (2.0f * fx);
+          const float t = (zeta >= 0.0f ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
+          const double td = (double)t;
+          cs = rsqrt(fma(td, td, 1.0));
+          sn = cs * td;
+        }
+      }
+      v = low ? cs * v - sn * w : sn * w + cs * v;
+    }
+    if (!__any_sync(0xffffffffu, more)) break;
+  }
+  if (lane < 16) sh.B[lane] = v;
+  else sh.J[lane - 16] = v;
+  double nn = v * v;
+  nn += __shfl_xor_sync(0xffffffffu, nn, 4);
+  nn += __shfl_xor_sync(0xffffffffu, nn, 8);
+  nn = __shfl_sync(0xffffffffu, nn, c);  // squared singular value of column c
+  double top = fmax(nn, __shfl_xor_sync(0xffffffffu, nn, 1));
+  top = fmax(top, __shfl_xor_sync(0xffffffffu, top, 2));
+  const bool full = __all_sync(0xffffffffu, nn > 1e-26 * top && nn > 0.0);
+  __syncwarp();
+  if (full) {
+    if (lane < 16) sh.B[lane] = v * rsqrt(nn);
+    __syncwarp();
+    double acc = 0.0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) acc = fma(sh.J[r * 4 + k], sh.B[c * 4 + k], acc);
+    if (lane < 16) sh.u[lane] = -acc;
+  } else if (lane == 0) {  // rank-deficient columns are completed by one thread
+    double G[16], u[16];
+    for (int i = 0; i < 16; ++i) G[i] = sh.g[i];
+    mera_solve(G, u);
+    for (int i = 0; i < 16; ++i) sh.u[i] = u[i];
+  }
+  __syncwarp();
+}
+
+__global__ void __launch_bounds__(32) de_mera_kernel(DEArgs a) {
+  __shared__ DeShared sh;
+  const int k = blockIdx.x, lane = threadIdx.x;
+  const int b0 = a.ent_begin[k], n = a.ent_begin[k + 1] - b0;
+  for (int e = lane; e < 16 * n; e += 32) {
+    sh.M[e >> 4][e & 15] = a.vals[a.ent_midx[16L * b0 + e]];
+    sh.C[e >> 4][e & 15] = a.ent_C[16L * b0 + e];
+  }
+  double u = 0.0;  // lanes 0 .. 15: the accepted disentangler
+  if (lane < 16) {
+    u = a.u_in[16L * k + lane];
+    sh.u[lane] = u;
+    sh.rho[lane] = a.vals[a.rho_idx[16L * k + lane]];
+  }
+  __syncwarp();
+  double e = de_energy_warp(sh, n);
+  if (lane == 0) a.e_out[2 * k] = e;
   for (int it = 0; it < a.max_iter; ++it) {
-    de_gamma(a, k, b0, b1, u, g);
-    mera_solve(g, un);
-    const double en = de_energy(a, b0, b1, un);
+    de_gamma_warp(sh, n, a.lambda[k]);
+    mera_solve_warp(sh);
+    const double en = de_energy_warp(sh, n);
     if (!(en <= e + 1e-14 * fmax(1.0, fabs(e)))) break;
     const bool done = fabs(en - e) <= a.rel_dev * fmax(fabs(e), 1e-300);
-    for (int i = 0; i < 16; ++i) u[i] = un[i];
+    if (lane < 16) u = sh.u[lane];
     e = en;
     if (done) break;
   }
-  for (int i = 0; i < 16; ++i) a.u_out[16L * k + i] = u[i];
-  a.e_out[2 * k + 1] = e;
+  if (lane < 16) a.u_out[16L * k + lane] = u;
+  if (lane == 0) a.e_out[2 * k + 1] = e;
 }
 
 // ---- Riemannian conjugate gradients on O(4) (Sec. 4.1.2): the true E_k(u) with u
@@ -838,7 +986,7 @@ double attn_state::de_update(const std::vector<int>* only) {
     a.u_in = d_uin.as<double>();
   }
   if (ctx->cfg.de_method == 1) de_rgd_kernel<<<(nS + 63) / 64, 64, 0, ctx->stream>>>(a);
-  else de_mera_kernel<<<(nS + 63) / 64, 64, 0, ctx->stream>>>(a);
+  else de_mera_kernel<<<nS, 32, 0, ctx->stream>>>(a);
   ctx->launches++;
   ATTN_CHECK_CUDA(cudaGetLastError());
   std::vector<double> uout(uin.size()), eo(2L * nS);
