@@ -78,6 +78,30 @@ __global__ void multi_dot_partial(const double* basis, int nvec, long V, int D, 
   }
 }
 
+// The same for many contiguous vectors at once: blockIdx.y is the vector, blockIdx.x its chunk.
+// (One block walking over 192 vectors with a barrier each took 210 us for 50 MB.)
+__global__ void __launch_bounds__(LT) many_dot_partial(const double* __restrict__ basis, int nvec, long V, long chunk,
+                                                       const double* __restrict__ w, double* part) {
+  __shared__ double sh[LT / 32];
+  const long e0 = blockIdx.x * chunk, e1 = e0 + chunk < V ? e0 + chunk : V;
+  const double* b = basis + (long)blockIdx.y * V;
+  double s0 = 0.0, s1 = 0.0;
+  long e = e0 + threadIdx.x;
+  for (; e + LT < e1; e += 2 * LT) {
+    s0 = fma(b[e], w[e], s0);
+    s1 = fma(b[e + LT], w[e + LT], s1);
+  }
+  if (e < e1) s0 = fma(b[e], w[e], s0);
+  const double s = warp_sum(s0 + s1);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int k = 0; k < LT / 32; ++k) t += sh[k];
+    part[(long)blockIdx.x * nvec + blockIdx.y] = t;
+  }
+}
+
 // out[i] = sum_b part[b][i] (fixed order); optionally accum[i] += out[i].
 __global__ void multi_dot_reduce(const double* part, int nb, int nvec, double* out, double* accum, const double* done) {
   if (done && *done != 0.0) return;
@@ -671,6 +695,18 @@ int fused_grid(long V) {
 
 void multi_dot_g(attn_ctx* ctx, const double* basis, int nvec, long V, int D, const double* w, double* out,
                  double* accum, const double* done) {
+  if (nvec >= 16 && nvec <= 65535 && !done && D == 0) {
+    // chunks of at least 4096 entries, about four blocks per SM
+    const long nc = std::max<long>(1, std::min<long>((V + 4095) / 4096, 4L * ctx->num_sms / nvec));
+    const long chunk = (V + nc - 1) / nc;
+    const int nb = (int)((V + chunk - 1) / chunk);
+    ctx->partials.reserve(sizeof(double) * (size_t)nb * nvec);
+    many_dot_partial<<<dim3(nb, nvec), LT, 0, ctx->stream>>>(basis, nvec, V, chunk, w, ctx->partials.as<double>());
+    multi_dot_reduce<<<nvec, LT, 0, ctx->stream>>>(ctx->partials.as<double>(), nb, nvec, out, accum, done);
+    ctx->launches += 2;
+    ATTN_CHECK_CUDA(cudaGetLastError());
+    return;
+  }
   const int nb = vgrid(V);
   ctx->partials.reserve(sizeof(double) * (size_t)nb * std::max(nvec, 1));
   multi_dot_partial<<<nb, LT, 0, ctx->stream>>>(basis, nvec, V, D, w, ctx->partials.as<double>(), done);
