@@ -46,6 +46,7 @@
 
 #include "gemm_tc.h"
 #include "heff.h"
+#include "heff_tc_small.h"
 #include "ozaki.h"
 #include "tc_ptx.h"
 
@@ -506,11 +507,12 @@ template <> __device__ __forceinline__ float to_operand<float>(double v) { retur
 // X01[c][a][b], X02[b][a][c], X12[a][b][c]. One block handles a 32 x 32 tile of
 // the (b, c) plane of one a: X02 and X12 rows are contiguous in c like x, and
 // the b <-> c transpose for X01 goes through shared memory, so every global
-// access is coalesced.
+// access is coalesced. z0 .. z2: FP32 outputs to be zeroed on the way (or null).
 constexpr int kTile = 32;
 
 template <class T>
-__global__ void prep_x_kernel(const double* __restrict__ x, int m0, int m1, int m2, T* x01, T* x02, T* x12) {
+__global__ void prep_x_kernel(const double* __restrict__ x, int m0, int m1, int m2, T* x01, T* x02, T* x12, float* z0,
+                              float* z1, float* z2) {
   __shared__ T t[kTile][kTile + 2];
   const int a = blockIdx.z, b0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
   for (int bb = threadIdx.y; bb < kTile; bb += blockDim.y) {
@@ -519,7 +521,11 @@ __global__ void prep_x_kernel(const double* __restrict__ x, int m0, int m1, int 
       const T v = to_operand<T>(x[((long)a * m1 + b) * m2 + c]);
       t[bb][threadIdx.x] = v;
       if (x02) x02[((long)b * m0 + a) * m2 + c] = v;
-      if (x12) x12[((long)a * m1 + b) * m2 + c] = v;
+      const long e = ((long)a * m1 + b) * m2 + c;
+      if (x12) x12[e] = v;
+      if (z0) z0[e] = 0.0f;
+      if (z1) z1[e] = 0.0f;
+      if (z2) z2[e] = 0.0f;
     }
   }
   if (!x01) return;
@@ -611,9 +617,37 @@ struct TcState {
   // of products ([tchunk][m2][m0][m1]) and the per-product kernel's maps and parameters
   int nt = 0, tchunk = 0;
   DevBuf t0, t1, t2, w;
+  // the kernel for links of at most 64, pair products and three-link ones (heff_tc_small.cu)
+  SmallTc *sm = nullptr, *smt = nullptr;
+  bool sm_ready = false;
   TcMaps tmaps;
   TcParams tprm;
   size_t es() const { return tf ? 4 : 2; }
+  TcState() = default;
+  TcState(const TcState&) = delete;
+  TcState& operator=(const TcState&) = delete;
+  ~TcState() {
+    delete sm;
+    delete smt;
+  }
+  void build_small(attn_heff* h) {
+    attn_ctx* ctx = h->ctx;
+    const int* m = h->m;
+    if (!sm) sm = new SmallTc();
+    sm->prm.nkinds = 0;
+    for (int k = 0; k < 3; ++k)
+      if (R[k])
+        sm->add_kind(tf, m[kPairP[k]], m[kPairQ[k]], m[kPairS[k]], R[k], m[kPairS[k]], x[k].p, a[k].p, b[k].p,
+                     y[k].as<float>(), false);
+    sm->cut(std::max(ctx->num_sms, 1), ctx->stream);
+    if (nt && nt <= tchunk) {
+      if (!smt) smt = new SmallTc();
+      smt->prm.nkinds = 0;
+      smt->add_kind(tf, m[0], m[1], m[2], nt, nt * m[2], w.p, t0.p, t1.p, y[0].as<float>(), true);
+      smt->cut(std::max(ctx->num_sms, 1), ctx->stream);
+    }
+    sm_ready = true;
+  }
   // Split every kind's product list f ways (at least 8 products per CTA) and lay out
   // the grid: one CTA per slice pair and product range.
   // f >= 1: split grid (products of a slice pair over f CTAs); f = 0: persistent form
@@ -756,6 +790,8 @@ static TcState* tc_build(attn_heff* h, bool tf) {
     t->t1 = std::move(old->t1);
     t->t2 = std::move(old->t2);
     t->w = std::move(old->w);
+    std::swap(t->sm, old->sm);
+    std::swap(t->smt, old->smt);
     delete old;
   }
   h->tc[tf ? 1 : 0] = t;
@@ -899,24 +935,44 @@ void attn_heff::apply_tc(const double* x, double* y, bool tf) {
   // consumer-side wait limit (a short one is how tests make the kernel give up)
   const int wl = ctx->cfg.wait_limit_log2;
   t->prm.wait = t->tprm.wait = (wl > 0) ? (1LL << std::min(wl, 62)) : attn::tc::kWaitCycles;
+  // links of at most 64 go to the kernel for narrow products, unless a grid form of the general one is
+  // asked for (measured there and beside it: heff_tc_small.cu)
+  const int sched = ctx->cfg.tc_schedule;
+  const bool small = sched == 0 && small_tc_fits(this);
+  if (small && !t->sm_ready) t->build_small(this);
+  float* zk[3];
+  for (int k = 0; k < 3; ++k) zk[k] = small && t->R[k] && t->sm->shared ? t->y[k].as<float>() : nullptr;
+  if (small && t->nt && !t->R[0]) zk[0] = t->y[0].as<float>();  // the three-link products add onto it
   // the kind buffers are indexed by pair kind k (0,1,2); kinds with no products pass null
   void* xk[3];
   for (int k = 0; k < 3; ++k) xk[k] = (t->R[k] || (k == 2 && t->nt)) ? t->x[k].p : nullptr;
   if (tf)
     prep_x_kernel<float><<<tile_grid(m), dim3(kTile, 8), 0, st>>>(x, m[0], m[1], m[2], static_cast<float*>(xk[0]),
-                                                                   static_cast<float*>(xk[1]), static_cast<float*>(xk[2]));
+                                                                   static_cast<float*>(xk[1]), static_cast<float*>(xk[2]), zk[0], zk[1],
+                                                                   zk[2]);
   else
     prep_x_kernel<__nv_bfloat16><<<tile_grid(m), dim3(kTile, 8), 0, st>>>(
         x, m[0], m[1], m[2], static_cast<__nv_bfloat16*>(xk[0]), static_cast<__nv_bfloat16*>(xk[1]),
-        static_cast<__nv_bfloat16*>(xk[2]));
+        static_cast<__nv_bfloat16*>(xk[2]), zk[0], zk[1], zk[2]);
   ctx->launches++;
   auto zero_split_outputs = [&]() {
     for (int k = 0; k < 3; ++k)
       if (t->R[k]) ATTN_CHECK_CUDA(cudaMemsetAsync(t->y[k].p, 0, sizeof(float) * (size_t)V, st));
   };
   const std::array<int, 7> key = {m[0], m[1], m[2], t->R[0], t->R[1], t->R[2], tf ? 1 : 0};
-  const int sched = ctx->cfg.tc_schedule;
-  if (t->grid > 0 && sched == 2) {
+  // algorithmic FLOPs of the pair products and the internal operators
+  double pair_fl = 0.0;
+  for (int k = 0; k < 3; ++k) pair_fl += (double)npair[k] * 2.0 * (m[kPairP[k]] + m[kPairQ[k]]) * V;
+  for (int s = 0; s < 3; ++s)
+    if (has_hint[s]) pair_fl += 2.0 * m[s] * V;
+  if (small) {
+    if (t->sm->prm.nkinds) {
+      ctx->prof_begin(0);
+      t->sm->launch(false, tf, t->prm.err, t->prm.wait, st);
+      ctx->prof_end(0, pair_fl);
+      ctx->launches++;
+    }
+  } else if (t->grid > 0 && sched == 2) {
     // persistent form requested
     if (!t->persistent || !t->tuned) t->set_split(0);
     t->tuned = true;
@@ -931,7 +987,7 @@ void attn_heff::apply_tc(const double* x, double* y, bool tf) {
     t->set_split(f);
     t->tuned = true;
   }
-  if (t->grid > 0 && !t->tuned) {
+  if (!small && t->grid > 0 && !t->tuned) {
     auto hit = ctx->tc_split_cache.find(key);
     double fl_all = 0.0;
     for (int k = 0; k < 3; ++k) fl_all += (double)t->R[k] * 2.0 * (m[kPairP[k]] + m[kPairQ[k]]) * V;
@@ -951,7 +1007,7 @@ void attn_heff::apply_tc(const double* x, double* y, bool tf) {
       ctx->tc_split_cache[key] = f;
     }
   }
-  if (t->grid > 0 && !t->tuned) {
+  if (!small && t->grid > 0 && !t->tuned) {
     // Autotuner: time the candidate product splits on this H_eff's real input and
     // keep the fastest (one-off per shape, product counts and operand type, at the
     // first tensor-core application).
@@ -986,16 +1042,11 @@ void attn_heff::apply_tc(const double* x, double* y, bool tf) {
     t->tuned = true;
     ctx->tc_split_cache[key] = best_f;
   }
-  if (t->grid > 0) {
-    // algorithmic FLOPs of this launch: the pair products and the internal operators
-    double fl = 0.0;
-    for (int k = 0; k < 3; ++k) fl += (double)npair[k] * 2.0 * (m[kPairP[k]] + m[kPairQ[k]]) * V;
-    for (int s = 0; s < 3; ++s)
-      if (has_hint[s]) fl += 2.0 * m[s] * V;
+  if (!small && t->grid > 0) {
     if (t->split_any()) zero_split_outputs();
     ctx->prof_begin(0);
     launch_sandwich(false, t, t->grid, t->maps, t->prm, st);
-    ctx->prof_end(0, fl);
+    ctx->prof_end(0, pair_fl);
     ctx->launches++;
   }
   if (t->nt > 0) {
@@ -1003,7 +1054,7 @@ void attn_heff::apply_tc(const double* x, double* y, bool tf) {
     // TN GEMM, then Y01[c] += A_r W_r[c] B_r^T on the per-product kernel
     const int P = m[0], Q = m[1], S = m[2];
     const size_t es = t->es();
-    if (!t->R[0]) ATTN_CHECK_CUDA(cudaMemsetAsync(t->y[0].p, 0, sizeof(float) * (size_t)V, st));
+    if (!t->R[0] && !small) ATTN_CHECK_CUDA(cudaMemsetAsync(t->y[0].p, 0, sizeof(float) * (size_t)V, st));
     for (int r0 = 0; r0 < t->nt; r0 += t->tchunk) {
       const int Rc = std::min(t->tchunk, t->nt - r0);
       TnOperand A;  // x as [a b][c]: rows P Q, K = S
@@ -1015,6 +1066,13 @@ void attn_heff::apply_tc(const double* x, double* y, bool tf) {
       g.M = P * Q; g.N = S; g.K = S; g.Bhi = Rc; g.Blo = 1; g.a_bhi = 0; g.b_bhi = 1;
       g.C = t->w.p; g.c_type = tf ? 3 : 1; g.c_rs = 1; g.c_cs = (long)P * Q; g.c_bhi = V;
       tn_gemm(ctx, A, B, g, t->err);
+      if (small && t->nt <= t->tchunk) {
+        ctx->prof_begin(0);
+        t->smt->launch(true, tf, t->prm.err, t->prm.wait, st);
+        ctx->prof_end(0, (double)Rc * 2.0 * (P + Q) * V);
+        ctx->launches++;
+        break;
+      }
       KindParams& kp = t->tprm.kind[0];
       kp.R = Rc;
       const int pairs = (S + 1) / 2;
