@@ -147,6 +147,8 @@ struct GemmF64 {
   bool split_ok = false;
 };
 void gemm_f64(attn_ctx* ctx, const GemmF64& g);
+// C = beta C + alpha times the sum of g.gsplit dense partial results [gsplit][batch][M][N], in order.
+void split_reduce_f64(attn_ctx* ctx, const GemmF64& g, const double* partials);
 // The same kernels launched on a bare stream (no context, no allocation).
 cudaError_t gemm_f64_stream(cudaStream_t stream, const GemmF64& g);
 cudaError_t fill_f64_stream(cudaStream_t stream, double* p, size_t n, double v);

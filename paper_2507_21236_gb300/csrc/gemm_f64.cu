@@ -301,6 +301,13 @@ void gemm_f64(attn_ctx* ctx, const GemmF64& g0) {
   ATTN_CHECK_CUDA(cudaGetLastError());
 }
 
+void split_reduce_f64(attn_ctx* ctx, const GemmF64& g, const double* partials) {
+  const size_t per = (size_t)g.Bhi * g.Blo * g.M * g.N;
+  split_reduce_kernel<<<grid_for(per), 256, 0, ctx->stream>>>(g, partials);
+  ctx->launches++;
+  ATTN_CHECK_CUDA(cudaGetLastError());
+}
+
 cudaError_t gemm_f64_stream(cudaStream_t stream, const GemmF64& g) {
   if (g.M <= 0 || g.N <= 0 || g.Bhi <= 0 || g.Blo <= 0) return cudaSuccess;
   return launch_gemm(stream, g);

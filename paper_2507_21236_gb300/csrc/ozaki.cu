@@ -477,32 +477,42 @@ __global__ void oz_exponent_kernel(OzView v, int* E, long estride) {
   }
 }
 
-// The same for views whose rows are contiguous (row stride 1): one thread per row,
-// 256 consecutive rows per block, so every K index reads 2 KB of consecutive memory
-// (the tiled kernel above reads 256 bytes per K index there, which wastes DRAM pages
-// when K is strided). Blocks split K into chunks; loads are unrolled four deep.
+// The same for views whose rows are contiguous (row stride 1): a thread per row and K index,
+// kx consecutive rows and 256 / kx K indices per block, so that a view of few rows (64 of a link
+// operator's contraction) fills the block too and every K index reads up to 2 KB of consecutive
+// memory (the tiled kernel above reads 256 bytes per K index there, which wastes DRAM pages when K is
+// strided). Blocks split K into chunks; loads are unrolled four deep.
 constexpr int kER = 256;
-__global__ void __launch_bounds__(kER) oz_exponent_rows_kernel(OzView v, int* E, long estride, long kchunk) {
-  const long r = (long)blockIdx.y * kER + threadIdx.x;
+__global__ void __launch_bounds__(kER) oz_exponent_rows_kernel(OzView v, int* E, long estride, long kchunk, int kx) {
+  __shared__ int sh[kER];
+  const int tx = threadIdx.x % kx, ty = threadIdx.x / kx, ky = kER / kx;
+  const long r = (long)blockIdx.y * kx + tx;
   const int batch = blockIdx.z, bh = batch / v.nblo, bl = batch % v.nblo;
   const long Kt = oz_kcount(v, bl), kbase = oz_kbase(v, bl);
   const long k0 = (long)blockIdx.x * kchunk, k1 = k0 + kchunk < Kt ? k0 + kchunk : Kt;
-  if (r >= v.rows) return;
   int em = kEmptyRow;
-  long k = k0;
-  for (; k + 4 <= k1; k += 4) {
-    long long b[4];
+  if (r < v.rows) {
+    long k = k0 + ty;
+    for (; k + 3 * ky < k1; k += 4 * ky) {
+      long long b[4];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) b[u] = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k + u)]);
+      for (int u = 0; u < 4; ++u) b[u] = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k + u * ky)]);
 #pragma unroll
-    for (int u = 0; u < 4; ++u)
-      if (b[u] & 0x7FFFFFFFFFFFFFFFll) em = max(em, exp_bits(b[u]));
+      for (int u = 0; u < 4; ++u)
+        if (b[u] & 0x7FFFFFFFFFFFFFFFll) em = max(em, exp_bits(b[u]));
+    }
+    for (; k < k1; k += ky) {
+      const long long b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k)]);
+      if (b & 0x7FFFFFFFFFFFFFFFll) em = max(em, exp_bits(b));
+    }
   }
-  for (; k < k1; ++k) {
-    const long long b = __double_as_longlong(v.p[oz_offset(v, bh, bl, r, kbase + k)]);
-    if (b & 0x7FFFFFFFFFFFFFFFll) em = max(em, exp_bits(b));
+  if (ky > 1) {
+    sh[threadIdx.x] = em;
+    __syncthreads();
+    if (ty == 0)
+      for (int h = 1; h < ky; ++h) em = max(em, sh[h * kx + tx]);
   }
-  if (em > kEmptyRow) atomicMax(&E[(long)batch * estride + r], em);
+  if (ty == 0 && r < v.rows && em > kEmptyRow) atomicMax(&E[(long)batch * estride + r], em);
 }
 
 // Slice s of 2^-E[row] entry, written tiled: element (batch, row, k) of slice s at
@@ -625,12 +635,14 @@ void ozaki_slice_to(attn_ctx* ctx, const OzView& v, long Kpad, int tile_rows, __
   ATTN_REQUIRE(rt <= 65535, ATTN_EUNSUPPORTED, "too many rows for the split GEMM");
   dim3 blk(kT, 8);
   if (v.sR == 1) {
-    // rows contiguous: one thread per row, K split into chunks for about 2048 blocks
-    const long rb = (v.rows + kER - 1) / kER;
-    const long nchunk = std::max<long>(1, std::min<long>((Kt + 63) / 64, 2048 / std::max<long>(rb * nb, 1)));
+    // rows contiguous: K split into chunks for about 2048 blocks, at least 16 K indices a thread
+    int kx = 32;
+    while (kx < kER && kx < v.rows) kx *= 2;
+    const long rb = (v.rows + kx - 1) / kx, per = 16L * (kER / kx);
+    const long nchunk = std::max<long>(1, std::min<long>((Kt + per - 1) / per, 2048 / std::max<long>(rb * nb, 1)));
     const long kchunk = (Kt + nchunk - 1) / nchunk;
     dim3 ge((unsigned)((Kt + kchunk - 1) / kchunk), (unsigned)rb, (unsigned)nb);
-    oz_exponent_rows_kernel<<<ge, kER, 0, st>>>(v, exps, exp_stride, kchunk);
+    oz_exponent_rows_kernel<<<ge, kER, 0, st>>>(v, exps, exp_stride, kchunk, kx);
   } else {
     // exponent pass: k tiles folded so that the grid stays modest
     const long kt = (Kt + kT - 1) / kT;
@@ -746,6 +758,20 @@ void gemm_f64_ozaki(attn_ctx* ctx, const GemmF64& g0) {
   const int gstep = std::max(1, (int)std::min<long>(g0.G, 65536L / std::max(g0.K, 1)));
   ATTN_REQUIRE(g0.K <= 65536, ATTN_EUNSUPPORTED, "K above 65536 for the split GEMM");
   oz_prepare(ctx);
+  // A product of few tiles over a long K (a link's renormalised operators: one 64 x 64 tile each)
+  // leaves SMs idle: its K goes to them in parts, batch entries of their own whose FP64 results are
+  // added up in order (all split GEMMs of an H_eff build at 16x16, m = 64: 42 -> 35 ms).
+  const long tiles0 = (long)((M + 127) / 128) * ((N + kQRows - 1) / kQRows) * g0.Bhi * g0.Blo;
+  const long Kall = (long)g0.K * g0.G;
+  long parts = 1;
+  if (g0.Blo == 1 && gstep >= g0.G && Kall >= 512)
+    parts = std::min<long>(std::max(ctx->num_sms, 1) / std::max<long>(tiles0, 1), Kall / 256);
+  if (parts > 1) {
+    const long kpart = (Kall + 64 * parts - 1) / (64 * parts) * 64;
+    P.kpart = Q.kpart = kpart;
+    P.nblo = Q.nblo = (int)((Kall + kpart - 1) / kpart);
+    P.sBlo = Q.sBlo = 0;
+  }
   const double fl = 2.0 * g0.M * g0.N * (double)g0.K * g0.G * g0.Bhi * g0.Blo;
   ctx->prof_begin(3);
   for (int ga = 0; ga < g0.G; ga += gstep) {
@@ -755,7 +781,7 @@ void gemm_f64_ozaki(attn_ctx* ctx, const GemmF64& g0) {
     q.p = Q.p + (long)ga * Q.sG;
     p.G = q.G = gn;
     const long Kt = (long)g0.K * gn;
-    const long Kpad = (Kt + 63) / 64 * 64;
+    const long Kpad = p.kpart ? p.kpart : (Kt + 63) / 64 * 64;
     ozaki_slice(ctx, p, Kpad, 128, ctx->oz_ws[0], ctx->oz_ws[1]);
     ozaki_slice(ctx, q, Kpad, kQRows, ctx->oz_ws[2], ctx->oz_ws[3]);
     const int nrtP = (M + 127) / 128, nrtQ = (N + kQRows - 1) / kQRows;
@@ -780,6 +806,25 @@ void gemm_f64_ozaki(attn_ctx* ctx, const GemmF64& g0) {
       prm.alpha_rest = pow2 ? (fr < 0 ? -1.0 : 1.0) : g0.alpha;
     }
     prm.beta = ga == 0 ? g0.beta : 1.0;
+    if (p.kpart) {
+      const long mn = (long)g0.M * g0.N, per = mn * g0.Bhi;
+      ctx->gsplit_ws.reserve(sizeof(double) * (size_t)p.nblo * per);
+      prm.Blo = p.nblo;
+      prm.p_lo = prm.q_lo = 1;
+      prm.C = ctx->gsplit_ws.as<double>();
+      prm.c_rs = swap ? 1 : g0.N;
+      prm.c_cs = swap ? g0.N : 1;
+      prm.c_bhi = mn;
+      prm.c_blo = per;
+      prm.alpha_exp = 0;
+      prm.alpha_rest = 1.0;
+      prm.beta = 0.0;
+      oz_launch(ctx, maps, prm);
+      GemmF64 r = g0;
+      r.gsplit = p.nblo;
+      split_reduce_f64(ctx, r, ctx->gsplit_ws.as<double>());
+      continue;
+    }
     oz_launch(ctx, maps, prm);
   }
   ctx->prof_end(3, fl);
