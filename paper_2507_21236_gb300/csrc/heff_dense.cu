@@ -511,7 +511,12 @@ __global__ void split_combine_kernel(double* __restrict__ y, int m0, int m1, int
   const int a = blockIdx.z, b0 = blockIdx.y * 32, c0 = blockIdx.x * 32;
   auto sum = [&](const double* p, int n, long at) {
     double v = p[at];
-    for (int i = 1; i < n; ++i) v += p[at + i * V];
+    int i = 1;
+    for (; i + 4 <= n; i += 4) {  // four loads in flight
+      const double a = p[at + i * V], b = p[at + (i + 1) * V], c = p[at + (i + 2) * V], d = p[at + (i + 3) * V];
+      v = (((v + a) + b) + c) + d;
+    }
+    for (; i < n; ++i) v += p[at + i * V];
     return v;
   };
   if (s.n[0]) {
