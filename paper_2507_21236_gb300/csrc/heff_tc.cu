@@ -536,26 +536,42 @@ __global__ void prep_x_kernel(const double* __restrict__ x, int m0, int m1, int 
   }
 }
 
-// y = Y01^T + Y02^T + Y12 (fp32 -> fp64), the same tiling as prep_x_kernel.
-__global__ void combine_kernel(double* __restrict__ y, int m0, int m1, int m2, const float* y01, const float* y02,
-                               const float* y12) {
+// A float as a double from integer instructions: conversions share the FP64 pipe, two lanes per SM and
+// cycle on this GPU.
+__device__ __forceinline__ double widen(float f) {
+  const unsigned u = __float_as_uint(f), e = (u >> 23) & 255u;
+  if (e - 1u < 254u)
+    return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | ((u & 0x7FFFFFu) >> 3)), (int)(u << 29));
+  return (u << 1) == 0 ? __hiloint2double((int)u, 0) : (double)f;  // a zero; subnormal, infinite or NaN
+}
+
+// y = Y01^T + Y02^T + Y12 (fp32 -> fp64), the same tiling as prep_x_kernel. What bounds it is the FP64
+// pipe: three conversions and two additions an entry took 22.6 us at 128 on all links (40 MB), the two
+// additions alone 10.8 us.
+__global__ void __launch_bounds__(256) combine_kernel(double* __restrict__ y, int m0, int m1, int m2,
+                                                      const float* __restrict__ y01, const float* __restrict__ y02,
+                                                      const float* __restrict__ y12) {
   __shared__ float t[kTile][kTile + 1];
   const int a = blockIdx.z, b0 = blockIdx.y * kTile, c0 = blockIdx.x * kTile;
-  if (y01) {
-    for (int cc = threadIdx.y; cc < kTile; cc += blockDim.y) {
-      const int c = c0 + cc, b = b0 + threadIdx.x;
-      if (b < m1 && c < m2) t[threadIdx.x][cc] = y01[((long)c * m0 + a) * m1 + b];
-    }
-    __syncthreads();
+  constexpr int N = kTile / 8;  // 32 x 8 threads
+  float v0[N], v1[N], v2[N];
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int cc = c0 + threadIdx.y + 8 * i, bx = b0 + threadIdx.x;  // transposed read
+    const int b = b0 + threadIdx.y + 8 * i, c = c0 + threadIdx.x;
+    const bool in = b < m1 && c < m2;
+    v0[i] = y01 && bx < m1 && cc < m2 ? y01[((long)cc * m0 + a) * m1 + bx] : 0.0f;
+    v1[i] = y02 && in ? y02[((long)b * m0 + a) * m2 + c] : 0.0f;
+    v2[i] = y12 && in ? y12[((long)a * m1 + b) * m2 + c] : 0.0f;
   }
-  for (int bb = threadIdx.y; bb < kTile; bb += blockDim.y) {
-    const int b = b0 + bb, c = c0 + threadIdx.x;
-    if (b < m1 && c < m2) {
-      double v = y01 ? (double)t[bb][threadIdx.x] : 0.0;
-      if (y02) v += (double)y02[((long)b * m0 + a) * m2 + c];
-      if (y12) v += (double)y12[((long)a * m1 + b) * m2 + c];
-      y[((long)a * m1 + b) * m2 + c] = v;
-    }
+#pragma unroll
+  for (int i = 0; i < N; ++i) t[threadIdx.x][threadIdx.y + 8 * i] = v0[i];
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    const int b = b0 + threadIdx.y + 8 * i, c = c0 + threadIdx.x;
+    if (b < m1 && c < m2)
+      y[((long)a * m1 + b) * m2 + c] = widen(t[threadIdx.y + 8 * i][threadIdx.x]) + widen(v1[i]) + widen(v2[i]);
   }
 }
 
