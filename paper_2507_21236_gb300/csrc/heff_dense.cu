@@ -16,8 +16,8 @@
 // With f64_split, M is held as its six BF16 slices (12 bytes per entry, written once), and an
 // application is one split GEMM per kind instead of two with a 1 GiB intermediate that has to be
 // sliced in between. Measured (GB300, one
-// application): [64]^3 with 140 products per pair 25.4 -> 5.6 ms; [16]^3 with 12
-// 128 -> 16 us, where the product-by-product path spends its time on 17 launches; f64_split at
+// application): [64]^3 with 140 products per pair 25.4 -> 5.5 ms; [16]^3 with 12
+// 128 -> 12 us, where the product-by-product path spends its time on 17 launches; f64_split at
 // [128]^3 with 288: 42.3 -> 3.5 ms (first application, which makes the slices: 42.7 -> 23.7 ms),
 // error against 64 bits 1.1e-13 -> 7.7e-14.
 #include <algorithm>
@@ -119,10 +119,8 @@ __device__ __forceinline__ void cp_async8(uint32_t dst, const double* src) {
 }
 
 constexpr int kDT = 256;      // threads
-constexpr int kDK = 32;       // K entries per step: one per lane of the loading warps
-constexpr int kDP = kDK + 1;  // padded row: the 32 rows a warp reads lie in different banks
 constexpr int kDStages = 3;
-constexpr int kDFold = 4;
+constexpr int kDFoldK = 128;  // K entries summed before they join the total
 
 // Shape of pair kind k in a TA x TB x TC block: rows (the block's extent along the pair,
 // second link fastest) and columns (along the remaining link).
@@ -137,9 +135,13 @@ struct DenseKind {
 // with x; blocks of fewer outputs than threads split every K step over G groups of threads,
 // whose sums meet at the end in a fixed order. Each loading warp takes every eighth row, so a
 // thread's rows are one pointer and one stride: with two warps per scheduler the integer work
-// of a step, not its copies, was what a small block waited for (24.6 -> 16.4 us at [16]^3).
-template <int TA, int TB, int TC>
+// of a step, not its copies, was what a small block waited for (24.6 -> 16.4 us at [16]^3; with 128 K entries a step 12.3 us).
+// HK: K entries per step and loading lane.
+template <int TA, int TB, int TC, int HK>
 struct DenseBlock {
+  static constexpr int kDK = 32 * HK;     // K entries per step
+  static constexpr int kDP = kDK + 1;     // padded row: the 32 rows a warp reads lie in different banks
+  static constexpr int kDFold = kDFoldK / kDK;
   static constexpr int OUT = TA * TB * TC;
   static constexpr int G = OUT < kDT ? kDT / OUT : 1;    // thread groups over K
   static constexpr int PER = OUT < kDT ? 1 : OUT / kDT;  // outputs per thread
@@ -197,26 +199,32 @@ struct DenseBlock {
   __device__ __forceinline__ void load(int s, int st) {
     using D = DenseKind<TA, TB, TC, k>;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int k0 = s * kDK, kg = k0 + lane;
-    const bool kin = kg < K[k];
+    const int k0 = s * kDK;
     double* Ms = sm + st * STAGE + w * kDP + lane;
-    const double* src = mp[k] + k0;
-#pragma unroll
-    for (int i = 0; i < D::ROWS / 8; ++i) copy(Ms + 8 * i * kDP, src + i * mstride[k], kin && i < live[k]);
     double* Xs = sm + st * STAGE + RMAX * kDP;
+    const double* src = mp[k] + k0;
     const int m1 = g.d[1], m2 = g.d[2];
+#pragma unroll
+    for (int h = 0; h < HK; ++h) {
+      const int kg = k0 + 32 * h + lane;
+      const bool kin = kg < K[k];
+#pragma unroll
+      for (int i = 0; i < D::ROWS / 8; ++i)
+        copy(Ms + 8 * i * kDP + 32 * h, src + 32 * h + i * mstride[k], kin && i < live[k]);
+      if (k > 0 && w < D::COLS) {
+        if (k == 1) {
+          const unsigned kp = (unsigned)kg / (unsigned)m2, kc = (unsigned)kg - kp * (unsigned)m2;
+          copy(Xs + w * kDP + 32 * h + lane, g.x + ((long)kp * m1 + b0 + w) * m2 + kc, kin && b0 + w < m1);
+        } else {
+          copy(Xs + w * kDP + 32 * h + lane, g.x + (long)(a0 + w) * K[2] + kg, kin && a0 + w < g.d[0]);
+        }
+      }
+    }
     if (k == 0) {  // x[k][c]: contiguous along the columns
 #pragma unroll
       for (int e = threadIdx.x; e < D::COLS * kDK; e += kDT) {
         const int c = e % TC, kk = e / TC, ke = k0 + kk;
         copy(Xs + c * kDP + kk, g.x + (long)ke * m2 + c0 + c, ke < K[0] && c0 + c < m2);
-      }
-    } else if (w < D::COLS) {
-      if (k == 1) {
-        const unsigned kp = (unsigned)kg / (unsigned)m2, kc = (unsigned)kg - kp * (unsigned)m2;
-        copy(Xs + w * kDP + lane, g.x + ((long)kp * m1 + b0 + w) * m2 + kc, kin && b0 + w < m1);
-      } else {
-        copy(Xs + w * kDP + lane, g.x + (long)(a0 + w) * K[2] + kg, kin && a0 + w < g.d[0]);
       }
     }
   }
@@ -249,7 +257,7 @@ struct DenseBlock {
 #pragma unroll
         for (int j = 0; j < PER; ++j) acc[j] = fma(mv, xc[j * CSTEP * kDP + q], acc[j]);
       }
-      // sums run over kDFold K steps before they join the total, so that rounding grows with
+      // sums run over kDFoldK entries before they join the total, so that rounding grows with
       // the root of that many terms and not of the whole row of M
       if (s % kDFold == kDFold - 1) {
 #pragma unroll
@@ -271,9 +279,9 @@ struct DenseBlock {
   }
 };
 
-template <int TA, int TB, int TC>
+template <int TA, int TB, int TC, int HK>
 __global__ void __launch_bounds__(kDT) dense_apply_kernel(const __grid_constant__ DenseApply g) {
-  using B = DenseBlock<TA, TB, TC>;
+  using B = DenseBlock<TA, TB, TC, HK>;
   extern __shared__ double sm[];
   double* ysum = sm + kDStages * B::STAGE;  // [G][OUT]
   B blk(g, sm);
@@ -294,18 +302,18 @@ __global__ void __launch_bounds__(kDT) dense_apply_kernel(const __grid_constant_
   }
 }
 
-template <int TA, int TB, int TC>
+template <int TA, int TB, int TC, int HK>
 void launch_dense(cudaStream_t st, const DenseApply& g) {
-  using B = DenseBlock<TA, TB, TC>;
+  using B = DenseBlock<TA, TB, TC, HK>;
   constexpr size_t smem = sizeof(double) * (kDStages * B::STAGE + B::G * B::OUT);
   static bool attr = false;  // (set again by a second thread: harmless)
   if (!attr) {
-    ATTN_CHECK_CUDA(cudaFuncSetAttribute(dense_apply_kernel<TA, TB, TC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    ATTN_CHECK_CUDA(cudaFuncSetAttribute(dense_apply_kernel<TA, TB, TC, HK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem));
     attr = true;
   }
   const long blocks = (long)((g.d[0] + TA - 1) / TA) * ((g.d[1] + TB - 1) / TB) * ((g.d[2] + TC - 1) / TC);
-  dense_apply_kernel<TA, TB, TC><<<(unsigned)blocks, kDT, smem, st>>>(g);
+  dense_apply_kernel<TA, TB, TC, HK><<<(unsigned)blocks, kDT, smem, st>>>(g);
 }
 
 // What the choices below weigh: the FP64 FMA rate that the kernels reach, a dependent launch
@@ -459,24 +467,32 @@ void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y
   }
   g.x = x;
   g.y = y;
-  // Block of y by the outputs that the busiest SM computes (FP64 FMAs bound the kernel),
-  // weighted by what a block shape loses to its loads; measured at 8 to 96 on all links, where
-  // the rule takes the fastest shape or one within 3 % of it.
+  // Block of y by the outputs that the busiest SM computes (FP64 FMAs bound the kernel), weighted by
+  // what a block shape loses to its loads, and K steps of 128 where they are not much padding, 64
+  // otherwise; measured at 8 to 96 on all links, where the rule takes the fastest or one within 5 %
+  // (16: 12.4 us against 16.5 with steps of 32; 32: 200 against 232; 64: 5.46 ms against 5.67).
   const long sms = std::max(ctx->num_sms, 1);
   const int* m = h->m;
   auto cost = [&](int ta, int tb, int tc, double weight) {
     const long blocks = (long)((m[0] + ta - 1) / ta) * ((m[1] + tb - 1) / tb) * ((m[2] + tc - 1) / tc);
     return weight * (double)((blocks + sms - 1) / sms * (ta * tb * tc));
   };
-  const double c[5] = {cost(8, 8, 8, 1.0), cost(4, 8, 8, 1.0), cost(4, 4, 8, 1.02), cost(4, 4, 4, 1.1),
-                       cost(4, 4, 2, 1.28)};
-  const int best = (int)(std::min_element(c, c + 5) - c);
+  const double c[3] = {cost(4, 4, 8, 1.0), cost(4, 4, 4, 1.01), cost(4, 4, 2, 1.06)};
+  const int best = (int)(std::min_element(c, c + 3) - c);
+  long K = 0, padded = 0;
+  for (int k = 0; k < 3; ++k)
+    if (g.m[k]) {
+      const long pq = (long)m[kPairP[k]] * m[kPairQ[k]];
+      K += pq;
+      padded += (pq + 127) / 128 * 128;
+    }
+  const bool wide = 10 * padded <= 11 * K;
   ctx->prof_begin(1);
-  if (best == 0) launch_dense<8, 8, 8>(ctx->stream, g);
-  else if (best == 1) launch_dense<4, 8, 8>(ctx->stream, g);
-  else if (best == 2) launch_dense<4, 4, 8>(ctx->stream, g);
-  else if (best == 3) launch_dense<4, 4, 4>(ctx->stream, g);
-  else launch_dense<4, 4, 2>(ctx->stream, g);
+  if (best == 0) launch_dense<4, 4, 8, 2>(ctx->stream, g);
+  else if (best == 1 && wide) launch_dense<4, 4, 4, 4>(ctx->stream, g);
+  else if (best == 1) launch_dense<4, 4, 4, 2>(ctx->stream, g);
+  else if (wide) launch_dense<4, 4, 2, 4>(ctx->stream, g);
+  else launch_dense<4, 4, 2, 2>(ctx->stream, g);
   ctx->prof_end(1, fl);
   ctx->launches++;
   ATTN_CHECK_CUDA(cudaGetLastError());
