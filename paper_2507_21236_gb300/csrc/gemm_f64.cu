@@ -8,7 +8,7 @@
 // shared-memory-tiled register-blocked GEMM: a BM x BN output tile per
 // 256-thread CTA (16 x 16 threads, BM/16 x BN/16 accumulators each), K tile 16;
 // loads pick the coalesced mapping from the unit stride of each operand. The
-// tile is 32 or 64 wide in each direction, chosen from M and N: the mode
+// tile is 16, 32 or 64 wide in each direction, chosen from M, N and the batch: the mode
 // products of link dimension 32 are batches of 32 x 32 GEMMs, which a 64 x 64
 // tile would compute at a quarter of its width. A GEMM whose output tiles do not
 // fill one wave of resident CTAs (the product-summing stage at m = 64 has 64)
@@ -194,14 +194,16 @@ static int sm_count() {
 // Tile of g: the one whose busiest SM computes the fewest outputs (FP64 FMAs at two per cycle
 // and SM bound the kernel). A batch too short for a tile per SM takes smaller ones:
 // the 64 x 4096 x 64 product of a centre move 69 -> 37 us with 64 x 32 tiles (128 instead of 64).
-// 5 % for the loads of a 32-wide side.
+// 5 % for the loads of a side below 64; 16 x 64 for the products of links of 16, which a 32-wide
+// tile would compute at half of its width.
 static void tile_of(const GemmF64& g, int* bm, int* bn) {
   const long nb = (long)g.Bhi * g.Blo * g.gsplit, sms = sm_count();
   double best = 0.0;
-  for (int m : {64, 32})
-    for (int n : {64, 32}) {
+  for (int m : {64, 32, 16})
+    for (int n : {64, 32, 16}) {
+      if (m * n < 16 * 64) continue;
       const long tiles = (long)((g.M + m - 1) / m) * ((g.N + n - 1) / n) * nb;
-      const double cost = (double)((tiles + sms - 1) / sms) * m * n * (m == 32 ? 1.05 : 1.0) * (n == 32 ? 1.05 : 1.0);
+      const double cost = (double)((tiles + sms - 1) / sms) * m * n * (m < 64 ? 1.05 : 1.0) * (n < 64 ? 1.05 : 1.0);
       if (best == 0.0 || cost < best) {
         best = cost;
         *bm = m;
@@ -214,12 +216,13 @@ static void tile_of(const GemmF64& g, int* bm, int* bn) {
 cudaError_t launch_gemm(cudaStream_t stream, const GemmF64& g) {
   int bm, bn;
   tile_of(g, &bm, &bn);
-  const bool sm = bm == 32, sn = bn == 32;
   dim3 grid((g.N + bn - 1) / bn, (g.M + bm - 1) / bm, (unsigned)std::min<long>((long)g.Bhi * g.Blo * g.gsplit, 65535));
   if (grid.y > 65535) return cudaErrorInvalidValue;
-  if (sm && sn) gemm_f64_kernel<32, 32><<<grid, NT, 0, stream>>>(g);
-  else if (sm) gemm_f64_kernel<32, 64><<<grid, NT, 0, stream>>>(g);
-  else if (sn) gemm_f64_kernel<64, 32><<<grid, NT, 0, stream>>>(g);
+  if (bm == 16) gemm_f64_kernel<16, 64><<<grid, NT, 0, stream>>>(g);
+  else if (bn == 16) gemm_f64_kernel<64, 16><<<grid, NT, 0, stream>>>(g);
+  else if (bm == 32 && bn == 32) gemm_f64_kernel<32, 32><<<grid, NT, 0, stream>>>(g);
+  else if (bm == 32) gemm_f64_kernel<32, 64><<<grid, NT, 0, stream>>>(g);
+  else if (bn == 32) gemm_f64_kernel<64, 32><<<grid, NT, 0, stream>>>(g);
   else gemm_f64_kernel<64, 64><<<grid, NT, 0, stream>>>(g);
   return cudaGetLastError();
 }
