@@ -1,6 +1,7 @@
 """Link operators renormalised in one launch (tensors of up to 4096 entries) against the oracle's
 sum of its per-product renormalised operators: dimensions that fill no block, the largest tensor
-that takes the one-launch path and the first that does not."""
+that takes the one-launch path, the first that does not (its one-sided products all go through the
+tensor pair) and one whose links have lists on both sides of that rule."""
 import numpy as np
 import pytest
 
@@ -9,7 +10,7 @@ from tests.test_gpu_boundary import _close, _pair
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("L,m,n_de", [(4, 3, 0), (4, 13, 4), (4, 16, 4), (8, 17, 16)])
+@pytest.mark.parametrize("L,m,n_de", [(4, 3, 0), (4, 13, 4), (4, 16, 4), (8, 17, 16), (8, 33, 16)])
 def test_internal_link_operators_match_oracle(L, m, n_de):
     attn, ctx, mod, st, ost, terms, tree, des, us = _pair(L, m, n_de)
     for node, slot in ((tree.top_nodes()[0], 0), (tree.top_nodes()[0], 2), (tree.node_id(2, 1), 1),
