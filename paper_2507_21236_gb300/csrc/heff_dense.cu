@@ -18,7 +18,7 @@
 // sliced in between. Measured (GB300, one
 // application): [64]^3 with 140 products per pair 25.4 -> 5.5 ms; [16]^3 with 12
 // 128 -> 12 us, where the product-by-product path spends its time on 17 launches; f64_split at
-// [128]^3 with 288: 42.3 -> 3.5 ms (first application, which makes the slices: 42.7 -> 23.7 ms),
+// [128]^3 with 288: 42.3 -> 3.4 ms (first application, which makes the slices: 42.7 -> 21.5 ms),
 // error against 64 bits 1.1e-13 -> 7.7e-14.
 #include <algorithm>
 #include <cmath>
@@ -594,54 +594,62 @@ DenseSplit* dense_split(attn_heff* h) {
   DenseSplit* d = h->dense_s;
   d->ctx = ctx;
   if (!dense_reserve(ctx, d->slices, need, d->bytes)) return nullptr;
-  d->exps.reserve(sizeof(int) * ne);
   bool hint_done[3] = {false, false, false};
-  for (int k = 0; k < 3; ++k) {
-    d->use[k] = use[k];
-    d->at[k] = at[k];
-    d->eat[k] = eat[k];
-    d->kpart[k] = kpart[k];
-    if (!use[k]) continue;
-    const int p = kPairP[k], q = kPairQ[k], P = h->m[p], Q = h->m[q], R = h->npair[k];
-    const long PQ = (long)P * Q, parts = (PQ + kpart[k] - 1) / kpart[k], tiles = (PQ + 127) / 128;
-    const long part_slices = tiles * (kpart[k] / 64) * 6 * 128 * 64;
-    const double* hp = h->has_hint[p] && !hint_done[p] ? h->hint[p].as<double>() : nullptr;
-    const double* hq = h->has_hint[q] && !hint_done[q] ? h->hint[q].as<double>() : nullptr;
-    hint_done[p] = hint_done[q] = true;
-    // values of the first link at a time: whole 128-row tiles of M, about kStage entries
-    int unit = 1;
-    while (unit < 128 && (unit * Q) % 128) ++unit;
-    const int step = (int)std::max<long>(1, std::min<long>(P, kStage / (PQ * Q)) / unit) * unit;
-    ctx->ws[0].reserve(sizeof(double) * (size_t)std::min(step, P) * Q * PQ);
-    double* stage = ctx->ws[0].as<double>();
-    for (int i0 = 0; i0 < P; i0 += step) {
-      const int i1 = std::min(P, i0 + step);
-      GemmF64 g;  // M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j'], a batch entry per (i, j)
-      g.split_ok = true;
-      g.M = P; g.N = Q; g.K = R;
-      g.Bhi = i1 - i0; g.Blo = Q;
-      g.A = h->pa[k].as<double>() + (long)i0 * P; g.aM = 1; g.aK = (long)P * P; g.aBhi = P;
-      g.B = h->pb[k].as<double>(); g.bN = 1; g.bK = (long)Q * Q; g.bBlo = Q;
-      g.C = stage; g.cM = Q; g.cN = 1; g.cBhi = Q * PQ; g.cBlo = PQ;
-      gemm_f64(ctx, g);
-      if (hp || hq) {
-        const long rows = (long)(i1 - i0) * Q;
-        add_internal_kernel<<<(int)std::min<long>((rows + 127) / 128, 4096), 128, 0, ctx->stream>>>(stage, P, Q, i0, i1,
-                                                                                                hp, hq);
-        ctx->launches++;
+  try {
+    d->exps.reserve(sizeof(int) * ne);
+    for (int k = 0; k < 3; ++k) {
+      d->use[k] = use[k];
+      d->at[k] = at[k];
+      d->eat[k] = eat[k];
+      d->kpart[k] = kpart[k];
+      if (!use[k]) continue;
+      const int p = kPairP[k], q = kPairQ[k], P = h->m[p], Q = h->m[q], R = h->npair[k];
+      const long PQ = (long)P * Q, parts = (PQ + kpart[k] - 1) / kpart[k], tiles = (PQ + 127) / 128;
+      const long part_slices = tiles * (kpart[k] / 64) * 6 * 128 * 64;
+      const double* hp = h->has_hint[p] && !hint_done[p] ? h->hint[p].as<double>() : nullptr;
+      const double* hq = h->has_hint[q] && !hint_done[q] ? h->hint[q].as<double>() : nullptr;
+      hint_done[p] = hint_done[q] = true;
+      // values of the first link at a time: whole 128-row tiles of M, about kStage entries
+      int unit = 1;
+      while (unit < 128 && (unit * Q) % 128) ++unit;
+      const int step = (int)std::max<long>(1, std::min<long>(P, kStage / (PQ * Q)) / unit) * unit;
+      ctx->ws[0].reserve(sizeof(double) * (size_t)std::min(step, P) * Q * PQ);
+      double* stage = ctx->ws[0].as<double>();
+      for (int i0 = 0; i0 < P; i0 += step) {
+        const int i1 = std::min(P, i0 + step);
+        GemmF64 g;  // M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j'], a batch entry per (i, j)
+        g.split_ok = true;
+        g.M = P; g.N = Q; g.K = R;
+        g.Bhi = i1 - i0; g.Blo = Q;
+        g.A = h->pa[k].as<double>() + (long)i0 * P; g.aM = 1; g.aK = (long)P * P; g.aBhi = P;
+        g.B = h->pb[k].as<double>(); g.bN = 1; g.bK = (long)Q * Q; g.bBlo = Q;
+        g.C = stage; g.cM = Q; g.cN = 1; g.cBhi = Q * PQ; g.cBlo = PQ;
+        gemm_f64(ctx, g);
+        if (hp || hq) {
+          const long rows = (long)(i1 - i0) * Q;
+          add_internal_kernel<<<(int)std::min<long>((rows + 127) / 128, 4096), 128, 0, ctx->stream>>>(stage, P, Q, i0, i1,
+                                                                                                  hp, hq);
+          ctx->launches++;
+        }
+        OzView v;
+        v.p = stage;
+        v.sR = PQ; v.sK = 1;
+        v.rows = (int)((i1 - i0) * Q);
+        v.K = (int)PQ;
+        v.kpart = kpart[k];
+        const long row0 = (long)i0 * Q;
+        auto* s = reinterpret_cast<__nv_bfloat16*>(d->slices.as<uint8_t>() + at[k]) +
+                  row0 / 128 * (kpart[k] / 64) * 6 * 128 * 64;
+        v.nblo = (int)parts;
+        ozaki_slice_to(ctx, v, kpart[k], 128, s, d->exps.as<int>() + eat[k] + row0, part_slices, PQ);
       }
-      OzView v;
-      v.p = stage;
-      v.sR = PQ; v.sK = 1;
-      v.rows = (int)((i1 - i0) * Q);
-      v.K = (int)PQ;
-      v.kpart = kpart[k];
-      const long row0 = (long)i0 * Q;
-      auto* s = reinterpret_cast<__nv_bfloat16*>(d->slices.as<uint8_t>() + at[k]) +
-                row0 / 128 * (kpart[k] / 64) * 6 * 128 * 64;
-      v.nblo = (int)parts;
-      ozaki_slice_to(ctx, v, kpart[k], 128, s, d->exps.as<int>() + eat[k] + row0, part_slices, PQ);
     }
+  } catch (const Error& e) {  // no memory for the exponents or the stage: product by product, as without M
+    if (e.status != ATTN_ENOMEM) throw;
+    d->slices.release();
+    ctx->dense_bytes -= d->bytes;
+    d->bytes = 0;
+    return nullptr;
   }
   for (int s = 0; s < 3; ++s) d->hint[s] = hint_done[s];
   ATTN_CHECK_CUDA(cudaGetLastError());

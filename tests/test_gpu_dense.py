@@ -98,3 +98,45 @@ def test_repeated_split_applications_match_products(shape, counts):
             assert np.all(got[5] == 0.0)
     attn.attn_heff_destroy(H)
     attn.attn_destroy(ctx)
+
+
+def test_split_application_without_memory_for_the_sums():
+    """A device allocator that refuses the slices (604 MB), their exponents (under 1 MB) or the
+    stage they are made in (134 MB): the application goes product by product as the first one did, bit
+    for bit, and takes the sums once memory is there."""
+    import torch
+    from paper_2507_21236_gb300 import attn as A_
+
+    refuse, refused = [0, 0], []
+
+    def alloc(n, device):
+        if refuse[0] <= n < refuse[1]:
+            refused.append(n)
+            return 0
+        return torch.cuda.caching_allocator_alloc(n, device)
+
+    shape, counts = (64, 64, 64), (60, 50, 55)
+    hint, pairs, _ = _problem(shape, counts, 0, 7)
+    x = dev(random_vector(shape, 100))
+    A_.attn_set_allocator(alloc, lambda p, n, device: torch.cuda.caching_allocator_delete(p))
+    try:
+        attn, ctx = lib_and_ctx({"f64_split": 1})
+        keep = [[None if h is None else dev(h) for h in hint], {k: (dev(a), dev(b)) for k, (a, b) in pairs.items()}]
+        H = attn.attn_heff_create(ctx, shape, *keep)
+        out = []
+        for sizes in ((0, 0), (1 << 29, 1 << 40), (0, 1 << 20), (130000000, 1 << 29), (0, 0)):
+            refuse[:] = sizes
+            refused.clear()
+            y = dev(np.full(shape, np.nan))
+            attn.attn_heff_apply(H, x, y, attn.ATTN_F64)
+            attn.attn_sync(ctx)
+            out.append(host(y))
+            assert bool(refused) == bool(refuse[1])
+        attn.attn_heff_destroy(H)
+        attn.attn_destroy(ctx)
+    finally:
+        A_.attn_set_allocator(None, None)
+    for y in out[1:4]:
+        assert np.array_equal(y, out[0])
+    assert np.abs(out[4] - out[0]).max() <= 1e-12 * np.abs(out[0]).max()
+    assert not np.array_equal(out[4], out[0])
