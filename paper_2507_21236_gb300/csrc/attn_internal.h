@@ -145,6 +145,9 @@ struct GemmF64 {
   long cS = 0;
   // the contraction may run as exact BF16 slice products when attn_config.f64_split is set
   bool split_ok = false;
+  // entry of A and of B of batch entry bh (device, Bhi each; null: entry bh); not with split_ok
+  const int* aIdx = nullptr;
+  const int* bIdx = nullptr;
 };
 void gemm_f64(attn_ctx* ctx, const GemmF64& g);
 // C = beta C + alpha times the sum of g.gsplit dense partial results [gsplit][batch][M][N], in order.
@@ -154,9 +157,9 @@ cudaError_t gemm_f64_stream(cudaStream_t stream, const GemmF64& g);
 cudaError_t fill_f64_stream(cudaStream_t stream, double* p, size_t n, double v);
 
 // out[r] = mat_r x_slot in[r or shared] for a [m0][m1][m2] tensor; mats is a
-// stack [R][m_s][m_s]; in_stride 0 shares one input, V for per-r inputs.
+// stack [R][m_s][m_s]; in_stride 0 shares one input, V for per-r inputs; transposed: mat_r^T.
 void mode_product_f64(attn_ctx* ctx, const int dims[3], int slot, const double* mats, int R,
-                      const double* in, long in_stride, double* out, double beta);
+                      const double* in, long in_stride, double* out, double beta, bool transposed = false);
 
 // Small helper kernels.
 void fill_f64(attn_ctx* ctx, double* p, size_t n, double v);

@@ -41,8 +41,8 @@ __global__ void __launch_bounds__(NT) gemm_f64_kernel(GemmF64 g) {
   for (long bz = blockIdx.z; bz < nb * g.gsplit; bz += gridDim.z) {
     const long sp = bz / nb, bb = bz % nb;
     const long bh = bb / g.Blo, bl = bb % g.Blo;
-    const double* Ab = g.A + bh * g.aBhi + bl * g.aBlo;
-    const double* Bb = g.B + bh * g.bBhi + bl * g.bBlo;
+    const double* Ab = g.A + (g.aIdx ? g.aIdx[bh] : bh) * g.aBhi + bl * g.aBlo;
+    const double* Bb = g.B + (g.bIdx ? g.bIdx[bh] : bh) * g.bBhi + bl * g.bBlo;
     double* Cb = g.C + sp * g.cS + bh * g.cBhi + bl * g.cBlo;
     const int ga = (int)(sp * g.G / g.gsplit), gb = (int)((sp + 1) * g.G / g.gsplit);
     double acc[TM][TN];
@@ -323,7 +323,7 @@ cudaError_t fill_f64_stream(cudaStream_t stream, double* p, size_t n, double v) 
 }
 
 void mode_product_f64(attn_ctx* ctx, const int d[3], int slot, const double* mats, int R, const double* in,
-                      long in_stride, double* out, double beta) {
+                      long in_stride, double* out, double beta, bool transposed) {
   const long V = (long)d[0] * d[1] * d[2];
   const long ms = (long)d[slot] * d[slot];
   GemmF64 g;
@@ -350,6 +350,10 @@ void mode_product_f64(attn_ctx* ctx, const int d[3], int slot, const double* mat
     g.B = mats; g.bK = 1; g.bN = d[2]; g.bBhi = ms;
     g.C = out; g.cM = d[2]; g.cN = 1; g.cBhi = V;
     g.Bhi = R; g.Blo = 1;
+  }
+  if (transposed) {
+    if (slot == 2) std::swap(g.bK, g.bN);
+    else std::swap(g.aM, g.aK);
   }
   gemm_f64(ctx, g);
 }

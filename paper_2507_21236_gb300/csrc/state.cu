@@ -50,11 +50,16 @@ __global__ void gram_err_kernel(const double* G, int k, double* out) {
   if (threadIdx.x == 0) *out = sh[0];
 }
 
-// out[r][i][j] = sum over the two other slots of T[.. i at t ..] * W_r[.. j at t ..]
-void contract_tt(attn_ctx* ctx, const double* T, const int d[3], int t, const double* W, int R, double* out) {
+// out[r][i][j] = sum over the two other slots of T[.. i at t ..] * W_r[.. j at t ..], or of
+// T_a(r) and W_b(r) for device lists a and b of R entries each
+void contract_tt(attn_ctx* ctx, const double* T, const int d[3], int t, const double* W, int R, double* out,
+                 const int* a = nullptr, const int* b = nullptr) {
   const long V = (long)d[0] * d[1] * d[2];
   GemmF64 g;
-  g.split_ok = true;
+  g.split_ok = !a;
+  g.aIdx = a;
+  g.bIdx = b;
+  g.aBhi = a ? V : 0;
   g.M = g.N = d[t];
   g.Bhi = R;
   g.C = out; g.cM = d[t]; g.cN = 1; g.cBhi = (long)d[t] * d[t];
@@ -359,6 +364,37 @@ void attn_state::renorm_batch(const double* Tc, const int d[3], int t, int x, in
       f.B = rw1.as<double>(); f.bK = osz; f.bN = 1;
       f.C = out; f.cM = osz; f.cN = 1;
       gemm_f64(ctx, f);
+      return;
+    }
+  }
+  if (!ia.empty() && !ib.empty() && !ctx->cfg.f64_split) {
+    // Lists that repeat their operators (the matrix units and terms of a disentangler's probes: 116 pairs of 20
+    // and 17, 192 of 28 and 28) take each operator once,
+    //     O_r = sum U_a(r) W_b(r),  U_a = A_a^T T on slot x,  W_b = B_b T on slot y,
+    // one contraction per pair and no mode product per pair. FP64 FMAs bound all of it, so the rule counts
+    // them; disentangler update of 8x8 at 32: 13.05 -> 11.4 ms.
+    std::vector<int> ua(ia), ub(ib);
+    for (auto* u : {&ua, &ub}) {
+      std::sort(u->begin(), u->end());
+      u->erase(std::unique(u->begin(), u->end()), u->end());
+    }
+    const int na = (int)ua.size(), nb = (int)ub.size();
+    if ((double)na * d[x] + (double)nb * d[y] < 0.9 * R * (d[x] + d[y]) && std::max(na, nb) <= chunk) {
+      std::vector<int> lists(ua);
+      lists.insert(lists.end(), ub.begin(), ub.end());
+      for (int i : ia) lists.push_back((int)(std::lower_bound(ua.begin(), ua.end(), i) - ua.begin()));
+      for (int i : ib) lists.push_back((int)(std::lower_bound(ub.begin(), ub.end(), i) - ub.begin()));
+      upload_idx(ctx, idxbuf, lists);
+      const int* dl = idxbuf.as<int>();
+      opsA.reserve(sizeof(double) * (size_t)na * d[x] * d[x]);
+      opsB.reserve(sizeof(double) * (size_t)nb * d[y] * d[y]);
+      rw1.reserve(sizeof(double) * (size_t)na * V);
+      rw2.reserve(sizeof(double) * (size_t)nb * V);
+      gather_rows_f64(ctx, opsA.as<double>(), Aops, dl, na, (long)d[x] * d[x]);
+      gather_rows_f64(ctx, opsB.as<double>(), Bops, dl + na, nb, (long)d[y] * d[y]);
+      mode_product_f64(ctx, d, x, opsA.as<double>(), na, Tc, 0, rw1.as<double>(), 0.0, true);
+      mode_product_f64(ctx, d, y, opsB.as<double>(), nb, Tc, 0, rw2.as<double>(), 0.0);
+      contract_tt(ctx, rw1.as<double>(), d, t, rw2.as<double>(), R, out, dl + na + nb, dl + na + nb + R);
       return;
     }
   }

@@ -5,7 +5,8 @@ tensor pair) and one whose links have lists on both sides of that rule."""
 import numpy as np
 import pytest
 
-from tests.test_gpu_boundary import _close, _pair
+from oracle.de_update import build_problems, rdms
+from tests.test_gpu_boundary import _close, _orth, _pair
 
 pytestmark = pytest.mark.gpu
 
@@ -34,4 +35,24 @@ def test_internal_link_operators_match_oracle(L, m, n_de):
         want = ost.heff_apply(nb, x)
         assert np.abs(y - want).max() <= 1e-12 * np.abs(want).max()
         attn.attn_heff_destroy(H)
+    _close(attn, ctx, mod, st)
+
+
+@pytest.mark.parametrize("m", [17, 24])
+def test_probe_lists_with_repeated_operators_match_oracle(m):
+    """Density matrices and environments at link dimensions above the one-launch path, where the
+    lists of probes open on two links repeat their operators; the boundary tests' bounds."""
+    attn, ctx, mod, st, ost, terms, tree, des, us = _pair(8, m, 16)
+    probs = build_problems(ost, terms, des)
+    ref = rdms(ost, [tuple(d) for d in des])
+    for k in range(len(des)):
+        assert np.abs(attn.attn_rdm2(st, k) - ref[k]).max() <= 1e-12, k
+        u = _orth(11, k)
+        g, e = attn.attn_de_environment(st, k, u)
+        gr, er = probs[k].gamma(u), probs[k].energy(u)
+        assert np.abs(g - gr).max() <= 1e-12 * max(1.0, np.abs(gr).max()), k
+        assert abs(e - er) <= 1e-12 * max(1.0, abs(er)), k
+    attn.attn_de_update(st)  # all at once: the longest lists
+    for p, u, e in zip(probs, us, attn.attn_de_energies(st, len(des))[:, 0]):
+        assert abs(e - p.energy(u)) <= 1e-12 * max(1.0, abs(e))
     _close(attn, ctx, mod, st)
