@@ -455,9 +455,12 @@ __global__ void __launch_bounds__(kQrT) qr_slab_kernel(const QrSlab q) {
         }
         for (int o = 16; o > 0; o >>= 1) fc += __shfl_xor_sync(0xffffffffu, fc, o);
         // c below 1e-9 of w, the usual case: its square is nothing beside |w|^2, and FP32 is enough
-        // for c . s, a correction of that size
+        // for c . s, a correction of that size, while both columns' norms lie where no term of it that
+        // matters leaves FP32's range
+        const double ny = y >= 0 ? sh.nrm0[y] : 1.0;
+        const bool mid = w2 > 1e-24 && w2 < 1e24 && ny > 1e-12 && ny < 1e12;
         double cc = 0.0, cs = 0.0;
-        if (fc <= 1e-18f) {
+        if (mid && fc <= 1e-18f) {
           float fs = 0.0f;
           for (int i = t; i < w && y >= 0; i += 32) fs = fmaf((float)sh.tot[i], (float)sh.tot[j + i], fs);
           for (int o = 16; o > 0; o >>= 1) fs += __shfl_xor_sync(0xffffffffu, fs, o);

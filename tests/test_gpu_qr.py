@@ -68,3 +68,32 @@ def test_dependent_columns_are_completed():
     attn.attn_state_destroy(st)
     attn.attn_model_destroy(mod)
     attn.attn_destroy(ctx)
+
+
+@pytest.mark.parametrize("even, odd", [(1e40, 1e40), (1e-40, 1e-40), (1e30, 1e-30), (1.0, 1e60)])
+def test_columns_outside_the_range_of_fp32(even, odd):
+    """Columns whose sums, or products of sums, FP32 cannot hold (the one-launch QR takes small corrections
+    in FP32); some of them nearly dependent, so that both Gram-Schmidt passes count."""
+    attn, ctx = lib_and_ctx()
+    m = 33
+    shapes = _shapes(m)
+    raw = [normal(8, n, int(np.prod(s))).reshape(s) for n, s in enumerate(shapes)]
+    mod = attn.attn_model_tfim(ctx, 4, 3.0)
+    st = attn.attn_state_create(ctx, mod, m, raw)
+    top, other = len(shapes) - 2, len(shapes) - 1
+    t = attn.attn_node_get(st, top)
+    t[:, :, 3::3] = t[:, :, :1] + 1e-7 * t[:, :, 3::3]
+    k = shapes[top][2]
+    t = t * np.where(np.arange(k) % 2 == 0, even, odd)[None, None, :]
+    attn.attn_node_set(st, top, t)
+    o = attn.attn_node_get(st, other)
+    before = np.einsum("abk,cdk->abcd", t, o)
+    attn.attn_move_centre(st, other)
+    q, c = attn.attn_node_get(st, top), attn.attn_node_get(st, other)
+    assert np.abs(np.einsum("abk,abl->kl", q, q) - np.eye(k)).max() < 1e-12
+    after = np.einsum("abk,cdk->abcd", q, c)
+    # backward error of a QR: a small multiple of k roundings of the tensor's norm
+    assert np.linalg.norm(after - before) <= 8 * k * 2.0 ** -53 * np.linalg.norm(before)
+    attn.attn_state_destroy(st)
+    attn.attn_model_destroy(mod)
+    attn.attn_destroy(ctx)
