@@ -48,11 +48,8 @@ struct PairOps {
 
 // M as a P^2 x Q^2 GEMM over the products (rows (i, i'), columns (j, j')); both operand
 // stacks are contiguous along the output index, so no transpose is needed. 64 x 64 tiles,
-// 4 x 4 per thread, 16 products per step. A step's products are summed by themselves before they join
-// the total (up to kBFew products, eight by eight): rounding then grows with the root of 16 products, not
-// of all. Error of an application at [64]^3 with 140 products 9.3e-16 -> 8.6e-16, FP64 pipe 97 % busy;
-// the sums of steps cost a twentieth of the first application (17.5 -> 18.4 ms, 25.4 product by product).
-constexpr int kBT = 64, kBK = 16, kBFew = 64;
+// 4 x 4 per thread, 16 products per step.
+constexpr int kBT = 64, kBK = 16;
 __global__ void __launch_bounds__(256) pair_operator_kernel(const PairOps ops) {
   __shared__ double As[kBK][kBT], Bs[kBK][kBT];
   int ki = 0;
@@ -63,20 +60,11 @@ __global__ void __launch_bounds__(256) pair_operator_kernel(const PairOps ops) {
   const int P2 = o.P * o.P, Q2 = o.Q * o.Q;
   const int i0 = (t / o.tiles_n) * kBT, j0 = (t % o.tiles_n) * kBT;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  double acc[4][4], tot[4][4];
+  double acc[4][4];
 #pragma unroll
   for (int i = 0; i < 4; ++i)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[i][j] = tot[i][j] = 0.0;
-  auto fold = [&]() {
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        tot[i][j] += acc[i][j];
-        acc[i][j] = 0.0;
-      }
-  };
+    for (int j = 0; j < 4; ++j) acc[i][j] = 0.0;
   for (int r0 = 0; r0 < o.R; r0 += kBK) {
 #pragma unroll
     for (int q = 0; q < kBK * kBT / 256; ++q) {
@@ -96,9 +84,7 @@ __global__ void __launch_bounds__(256) pair_operator_kernel(const PairOps ops) {
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
-      if (r == kBK / 2 - 1 && o.R <= kBFew) fold();
     }
-    fold();
     __syncthreads();
   }
   const long PQ = (long)o.P * o.Q;
@@ -112,7 +98,7 @@ __global__ void __launch_bounds__(256) pair_operator_kernel(const PairOps ops) {
       const int gj = j0 + tx + 16 * j;
       if (gj >= Q2) continue;
       const int q = gj / o.Q, qq = gj % o.Q;
-      double v = tot[i][j];
+      double v = acc[i][j];
       if (o.hp && q == qq) v += o.hp[gi];
       if (o.hq && p == pp) v += o.hq[gj];
       o.m[((long)p * o.Q + q) * PQ + (long)pp * o.Q + qq] = v;
@@ -308,14 +294,9 @@ __global__ void __launch_bounds__(kDT) dense_apply_kernel(const __grid_constant_
   blk.template run<2>(at, st, ysum);
   __syncthreads();
   for (int o = threadIdx.x; o < B::OUT; o += kDT) {
-    double part[B::G];
+    double v = ysum[o];
 #pragma unroll
-    for (int q = 0; q < B::G; ++q) part[q] = ysum[q * B::OUT + o];
-#pragma unroll
-    for (int w = B::G / 2; w > 0; w /= 2)
-#pragma unroll
-      for (int q = 0; q < w; ++q) part[q] += part[q + w];
-    const double v = part[0];
+    for (int q = 1; q < B::G; ++q) v += ysum[q * B::OUT + o];
     const int a = blk.a0 + o / (TB * TC), b = blk.b0 + o / TC % TB, c = blk.c0 + o % TC;
     if (a < g.d[0] && b < g.d[1] && c < g.d[2]) g.y[((long)a * g.d[1] + b) * g.d[2] + c] = v;
   }
@@ -344,7 +325,7 @@ constexpr double kF64Rate = 1.1e12, kLaunch = 4e-6, kAlloc = 5e-5;
 // Device memory for dense operators: at most a sixteenth of the GPU per context and, for more
 // than 64 MB at once, at most a quarter of what is free, so that programs with many handles or
 // a pool of their own keep the product-by-product path instead of running out. False when
-// there is no room (a buffer that could not grow is then empty and no longer counted).
+// there is no room (buf is then empty and no longer counted).
 bool dense_reserve(attn_ctx* ctx, DevBuf& buf, size_t n, size_t& counted) {
   if (n <= buf.bytes) return true;
   bool ok = ctx->dense_bytes - counted + n <= ctx->total_mem / 16;
