@@ -248,9 +248,8 @@ __device__ void de_gamma_warp(DeShared& sh, int n, double lambda) {
 
 // u = -V W^T for G = W diag(s) V^T (G in sh.g, u into sh.u): one-sided Jacobi on the columns of
 // G, two rotations at a time. Lane (m, r, c) holds entry (r, c) of B (m = 0) or of the
-// accumulated rotations J (m = 1). The angle comes from FP32 (any angle that reduces the
-// product of the columns will do, and the last sweeps take it to rounding), its cosine and sine
-// from FP64, so the rotations stay orthogonal.
+// accumulated rotations J (m = 1). The angle comes from FP32, which leaves 1e-7 of the columns'
+// product to the next sweep, its cosine and sine from FP64, so the rotations stay orthogonal.
 __device__ void mera_solve_warp(DeShared& sh) {
   const int lane = threadIdx.x & 31, r = (lane >> 2) & 3, c = lane & 3;
   double v = lane < 16 ? sh.g[lane] : (r == c ? 1.0 : 0.0);
@@ -283,8 +282,11 @@ __device__ void mera_solve_warp(DeShared& sh) {
         rot = ratio > 1e-16f * sqrtf(fminf(fa, fb));
         more = more || ratio > 1e-15f * sqrtf(fminf(fa, fb));
         if (rot && fx != 0.0f) {
-          const float zeta = (fb - fa) / (2.0f * fx);
-          const float t = (zeta >= 0.0f ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
+          // the difference in FP64: of nearly equal norms FP32 would leave nothing, and turning by
+          // 45 degrees then swaps x and the difference for ever
+          const float zeta = (float)((b - a) * sc) / (2.0f * fx);
+          const float t = fabsf(zeta) > 1e9f ? 0.5f / zeta  // (its square may leave FP32's range)
+                                             : (zeta >= 0.0f ? 1.0f : -1.0f) / (fabsf(zeta) + sqrtf(1.0f + zeta * zeta));
           const double td = (double)t;
           cs = rsqrt(fma(td, td, 1.0));
           sn = cs * td;
