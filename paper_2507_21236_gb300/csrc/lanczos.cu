@@ -701,13 +701,14 @@ __global__ void __launch_bounds__(kTailT) lz_tail_kernel(const LzTail<T> q) {
   }
   cg::cluster_group cl = cg::this_cluster();
   const int rank = (int)cl.block_rank(), n = q.k + 1, el = q.el;
-  // the second cluster may be setting the flag: one CTA reads it for all
-  if (rank == 0 && t < kTailC) {
-    const int d = *(volatile double*)(S + S_DONE) != 0.0;
-    *cl.map_shared_rank(&stop, t) = __shfl_sync((1u << kTailC) - 1u, d, 0);
-  }
+  // the second cluster may be setting the flag: one CTA reads it for all, which take it from there
+  // (after the barrier: before it a CTA of the cluster may not have started)
+  if (rank == 0 && t == 0) stop = *(volatile double*)(S + S_DONE) != 0.0;
   cl.sync();
-  if (stop) return;
+  if (*cl.map_shared_rank(&stop, 0)) {
+    cl.sync();
+    return;
+  }
   const long e0 = (long)rank * el;
   const int cnt = (int)max(0L, min((long)el, q.V - e0));
   T* sw = reinterpret_cast<T*>(tail_smem);  // w
