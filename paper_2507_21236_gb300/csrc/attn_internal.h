@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "attn.h"
+#include "per_device.h"
 
 namespace attn {
 
@@ -36,6 +37,12 @@ struct Error {
   do {                                                                                         \
     if (!(cond)) throw ::attn::Error{status, std::string(msg)};                                \
   } while (0)
+
+inline int current_device() {
+  int d = 0;
+  ATTN_CHECK_CUDA(cudaGetDevice(&d));
+  return d;
+}
 
 // ------------------------------------------------------------ device memory
 // Owning device buffer (cudaMalloc / cudaFree). A buffer that captured CUDA graphs

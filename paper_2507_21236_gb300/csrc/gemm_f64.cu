@@ -183,12 +183,13 @@ inline int grid_for(size_t n, int threads = 256, int cap = 4096) {
 }  // namespace
 
 static int sm_count() {
-  static int sms = 0;
-  int dev = 0, n = 0;
-  if (!sms && cudaGetDevice(&dev) == cudaSuccess &&
-      cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess)
-    sms = n;
-  return std::max(sms, 1);
+  static PerDevice sms;
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+  return sms.get(dev, [dev] {
+    int n = 0;
+    return cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) == cudaSuccess ? std::max(n, 1) : 1;
+  });
 }
 
 // Tile of g: the one whose busiest SM computes the fewest outputs (FP64 FMAs at two per cycle

@@ -172,12 +172,12 @@ void tn_gemm(attn_ctx* ctx, const TnOperand& A, const TnOperand& B, TnParams p, 
   err.reserve(sizeof(int));
   p.err = err.as<int>();
   const size_t smem = 1024 + (size_t)kStages * kStageBytes + 256;
-  static bool attr = false;
-  if (!attr) {
+  static PerDevice attr;
+  attr.get(current_device(), [smem] {
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(tn_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(tn_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-    attr = true;
-  }
+    return 1;
+  });
   const long total = (long)p.Bhi * p.Blo;
   dim3 grid((p.N + 127) / 128, (p.M + 127) / 128, 1);
   ATTN_REQUIRE(grid.y <= 65535, ATTN_EUNSUPPORTED, "GEMM M too large");

@@ -306,12 +306,12 @@ template <int TA, int TB, int TC, int HK>
 void launch_dense(cudaStream_t st, const DenseApply& g) {
   using B = DenseBlock<TA, TB, TC, HK>;
   constexpr size_t smem = sizeof(double) * (kDStages * B::STAGE + B::G * B::OUT);
-  static bool attr = false;  // (set again by a second thread: harmless)
-  if (!attr) {
+  static PerDevice attr;
+  attr.get(current_device(), [] {
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(dense_apply_kernel<TA, TB, TC, HK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)smem));
-    attr = true;
-  }
+    return 1;
+  });
   const long blocks = (long)((g.d[0] + TA - 1) / TA) * ((g.d[1] + TB - 1) / TB) * ((g.d[2] + TC - 1) / TC);
   dense_apply_kernel<TA, TB, TC, HK><<<(unsigned)blocks, kDT, smem, st>>>(g);
 }

@@ -437,14 +437,14 @@ void SmallTc::cut(int sms, cudaStream_t st) {
 void SmallTc::launch(bool pp, bool tf, int* err, long long wait, cudaStream_t st) {
   prm.err = err;
   prm.wait = wait;
-  static bool attr = false;  // (set again by a second thread: harmless)
-  if (!attr) {
+  static PerDevice attr;
+  attr.get(current_device(), [] {
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(small_tc_kernel<false, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(false, false)));
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(small_tc_kernel<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(false, true)));
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(small_tc_kernel<true, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(true, false)));
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(small_tc_kernel<true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_of(true, true)));
-    attr = true;
-  }
+    return 1;
+  });
   const size_t smem = smem_of(pp, tf);
   if (tf) {
     if (pp) small_tc_kernel<true, true><<<grid, kThreads, smem, st>>>(maps->m, prm);

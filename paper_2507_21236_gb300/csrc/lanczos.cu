@@ -790,12 +790,11 @@ __global__ void __launch_bounds__(kTailT) lz_tail_kernel(const LzTail<T> q) {
 // Entries per CTA if steps against up to `depth` vectors fit, else 0.
 template <class T>
 int tail_entries(long V, int depth) {
-  static int ok = -1;  // whether this GPU runs the cluster
   if (V > (long)kTailC * 8192 || depth > kTailN) return 0;
   const int el = (int)((V + kTailC - 1) / kTailC);
   if (sizeof(T) * (size_t)el * (depth + 1) > kTailSmem) return 0;
-  if (ok < 0) {
-    ok = 0;
+  static PerDevice runs;  // whether the GPU runs the cluster
+  const int ok = runs.get(current_device(), [] {
     cudaLaunchConfig_t c = {};
     c.gridDim = dim3(2 * kTailC);
     c.blockDim = dim3(kTailT);
@@ -807,12 +806,13 @@ int tail_entries(long V, int depth) {
     c.attrs = &attr;
     c.numAttrs = 1;
     int nc = 0;
-    if (cudaFuncSetAttribute(lz_tail_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem) == cudaSuccess &&
+    const bool fits =
+        cudaFuncSetAttribute(lz_tail_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmem) == cudaSuccess &&
         cudaFuncSetAttribute(lz_tail_kernel<T>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-        cudaOccupancyMaxActiveClusters(&nc, lz_tail_kernel<T>, &c) == cudaSuccess && nc >= 1)
-      ok = 1;
+        cudaOccupancyMaxActiveClusters(&nc, lz_tail_kernel<T>, &c) == cudaSuccess && nc >= 1;
     (void)cudaGetLastError();
-  }
+    return fits ? 1 : 0;
+  });
   return ok ? el : 0;
 }
 

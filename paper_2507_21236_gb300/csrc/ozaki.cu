@@ -693,11 +693,11 @@ namespace {
 constexpr size_t kOzSmem = 1024 + 2 * (size_t)kQBufBytes + (size_t)kPStages * kPBytes + 256;
 
 void oz_prepare(attn_ctx* ctx) {
-  static bool attr = false;
-  if (!attr) {
+  static PerDevice attr;
+  attr.get(current_device(), [] {
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(ozaki_gemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kOzSmem));
-    attr = true;
-  }
+    return 1;
+  });
   ctx->oz_err.reserve(sizeof(int));
   if (!ctx->oz_err_init) {
     ATTN_CHECK_CUDA(cudaMemsetAsync(ctx->oz_err.p, 0, sizeof(int), ctx->stream));

@@ -589,8 +589,8 @@ void qr_tensor(attn_ctx* ctx, double* T, const int d[3], int slot, double* R, QR
   QrSlab q;
   q.ld = k | 1;
   constexpr size_t kSmemMax = 200 * 1024;
-  static int most = 0;  // clusters that are resident together with a full slab per SM
-  if (!most) {
+  static PerDevice clusters;  // that are resident together with a full slab per SM
+  const int most = clusters.get(current_device(), [] {
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(qr_slab_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemMax));
     cudaLaunchConfig_t c = {};
     c.gridDim = dim3(kQrC);
@@ -604,8 +604,8 @@ void qr_tensor(attn_ctx* ctx, double* T, const int d[3], int slot, double* R, QR
     c.numAttrs = 1;
     int nc = 0;
     ATTN_CHECK_CUDA(cudaOccupancyMaxActiveClusters(&nc, qr_slab_kernel, &c));
-    most = std::max(nc, 1);
-  }
+    return std::max(nc, 1);
+  });
   // Clusters by the cycles of a column: rows x k FP64 FMAs at two per cycle on the busiest SM
   // (both passes, both products), the cluster barriers and, with more than one cluster, the grid
   // barrier and the sums over the clusters (measured around 3 us).

@@ -173,11 +173,11 @@ void renorm_small(attn_ctx* ctx, const double* T, const int d[3], int t, int x, 
   const long osz = (long)d[t] * d[t];
   const int groups_all = ((int)closed.size() + kGroup - 1) / kGroup;
   if (groups_all) part.reserve(sizeof(double) * groups_all * osz);
-  static bool attr = false;  // (set again by a second thread: harmless)
-  if (!attr) {
+  static PerDevice attr;
+  attr.get(current_device(), [] {
     ATTN_CHECK_CUDA(cudaFuncSetAttribute(renorm_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMaxSmem));
-    attr = true;
-  }
+    return 1;
+  });
   size_t io = 0, ic = 0;
   int groups_done = 0;
   while (io < open.size() || ic < closed.size()) {
