@@ -501,12 +501,12 @@ void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y
 // ---------------------------------------------------------------- as BF16 slices
 namespace {
 
-// M += H_p (x) 1 and 1 (x) H_q (either may be null) on the rows (i, j), i0 <= i < i1, that m
+// M += H_p (x) 1 and 1 (x) H_q (either may be null) on the rows r0 <= i Q + j < r1 that m
 // holds; one thread per row, since both add to the row's diagonal entry.
-__global__ void add_internal_kernel(double* m, int P, int Q, int i0, int i1, const double* hp, const double* hq) {
+__global__ void add_internal_kernel(double* m, int P, int Q, long r0, long r1, const double* hp, const double* hq) {
   const long PQ = (long)P * Q;
-  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < (long)(i1 - i0) * Q; e += (long)gridDim.x * blockDim.x) {
-    const int i = i0 + (int)(e / Q), j = (int)(e % Q);
+  for (long e = blockIdx.x * (long)blockDim.x + threadIdx.x; e < r1 - r0; e += (long)gridDim.x * blockDim.x) {
+    const int i = (int)((r0 + e) / Q), j = (int)((r0 + e) % Q);
     double* row = m + e * PQ;
     if (hp)
       for (int ii = 0; ii < P; ++ii) row[(long)ii * Q + j] += hp[(long)i * P + ii];
@@ -560,6 +560,18 @@ __global__ void split_combine_kernel(double* __restrict__ y, int m0, int m1, int
 constexpr double kSplitProd = 25e-12, kSplitMake = 20e-12, kSplitUse = 1.4e-12, kSplitKind = 5e-5;
 constexpr long kStage = 1L << 27;  // doubles of M made at a time (1 GiB)
 
+// Rows of M made at a time: whole 128-row tiles within the stage, and where that goes whole values of the
+// first link as well (one GEMM per stage). Where it does not (a second link with few factors of two:
+// 113 x 113 would take all of M, 1.3 GB, 191 x 191 7 GB) tiles alone.
+long stage_rows(int P, int Q) {
+  const long PQ = (long)P * Q;
+  int unit = 1;
+  while (unit < 128 && (unit * Q) % 128) ++unit;
+  const long step = std::max<long>(1, std::min<long>(P, kStage / (PQ * Q)) / unit) * unit;
+  if (std::min<long>(step, P) * Q * PQ <= kStage) return step * Q;
+  return std::max<long>(1, kStage / PQ / 128) * 128;
+}
+
 }  // namespace
 
 DenseSplit* dense_split(attn_heff* h) {
@@ -609,39 +621,42 @@ DenseSplit* dense_split(attn_heff* h) {
       const double* hp = h->has_hint[p] && !hint_done[p] ? h->hint[p].as<double>() : nullptr;
       const double* hq = h->has_hint[q] && !hint_done[q] ? h->hint[q].as<double>() : nullptr;
       hint_done[p] = hint_done[q] = true;
-      // values of the first link at a time: whole 128-row tiles of M, about kStage entries
-      int unit = 1;
-      while (unit < 128 && (unit * Q) % 128) ++unit;
-      const int step = (int)std::max<long>(1, std::min<long>(P, kStage / (PQ * Q)) / unit) * unit;
-      ctx->ws[0].reserve(sizeof(double) * (size_t)std::min(step, P) * Q * PQ);
+      const long rows = stage_rows(P, Q);
+      ctx->ws[0].reserve(sizeof(double) * (size_t)std::min(rows, PQ) * PQ);
       double* stage = ctx->ws[0].as<double>();
-      for (int i0 = 0; i0 < P; i0 += step) {
-        const int i1 = std::min(P, i0 + step);
-        GemmF64 g;  // M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j'], a batch entry per (i, j)
-        g.split_ok = true;
-        g.M = P; g.N = Q; g.K = R;
-        g.Bhi = i1 - i0; g.Blo = Q;
-        g.A = h->pa[k].as<double>() + (long)i0 * P; g.aM = 1; g.aK = (long)P * P; g.aBhi = P;
-        g.B = h->pb[k].as<double>(); g.bN = 1; g.bK = (long)Q * Q; g.bBlo = Q;
-        g.C = stage; g.cM = Q; g.cN = 1; g.cBhi = Q * PQ; g.cBlo = PQ;
-        gemm_f64(ctx, g);
+      for (long r0 = 0; r0 < PQ; r0 += rows) {
+        const long r1 = std::min(PQ, r0 + rows);
+        // M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j'], a batch entry per (i, j): all whole i at once,
+        // the part of one at either end
+        for (long r = r0; r < r1;) {
+          const int i = (int)(r / Q), j = (int)(r % Q);
+          const bool whole = j == 0 && r1 - r >= Q;
+          GemmF64 g;
+          g.split_ok = true;
+          g.M = P; g.N = Q; g.K = R;
+          g.Bhi = whole ? (int)((r1 - r) / Q) : 1;
+          g.Blo = whole ? Q : (int)std::min<long>(Q - j, r1 - r);
+          g.A = h->pa[k].as<double>() + (long)i * P; g.aM = 1; g.aK = (long)P * P; g.aBhi = P;
+          g.B = h->pb[k].as<double>() + (long)j * Q; g.bN = 1; g.bK = (long)Q * Q; g.bBlo = Q;
+          g.C = stage + (r - r0) * PQ; g.cM = Q; g.cN = 1; g.cBhi = Q * PQ; g.cBlo = PQ;
+          gemm_f64(ctx, g);
+          r += (long)g.Bhi * g.Blo;
+        }
         if (hp || hq) {
-          const long rows = (long)(i1 - i0) * Q;
-          add_internal_kernel<<<(int)std::min<long>((rows + 127) / 128, 4096), 128, 0, ctx->stream>>>(stage, P, Q, i0, i1,
-                                                                                                  hp, hq);
+          add_internal_kernel<<<(int)std::min<long>((r1 - r0 + 127) / 128, 4096), 128, 0, ctx->stream>>>(stage, P, Q, r0, r1,
+                                                                                                     hp, hq);
           ctx->launches++;
         }
         OzView v;
         v.p = stage;
         v.sR = PQ; v.sK = 1;
-        v.rows = (int)((i1 - i0) * Q);
+        v.rows = (int)(r1 - r0);
         v.K = (int)PQ;
         v.kpart = kpart[k];
-        const long row0 = (long)i0 * Q;
         auto* s = reinterpret_cast<__nv_bfloat16*>(d->slices.as<uint8_t>() + at[k]) +
-                  row0 / 128 * (kpart[k] / 64) * 6 * 128 * 64;
+                  r0 / 128 * (kpart[k] / 64) * 6 * 128 * 64;
         v.nblo = (int)parts;
-        ozaki_slice_to(ctx, v, kpart[k], 128, s, d->exps.as<int>() + eat[k] + row0, part_slices, PQ);
+        ozaki_slice_to(ctx, v, kpart[k], 128, s, d->exps.as<int>() + eat[k] + r0, part_slices, PQ);
       }
     }
   } catch (const Error& e) {  // no memory for the exponents or the stage: product by product, as without M
