@@ -325,7 +325,8 @@ constexpr double kF64Rate = 1.1e12, kLaunch = 4e-6, kAlloc = 5e-5;
 // Device memory for dense operators: at most a sixteenth of the GPU per context and, for more
 // than 64 MB at once, at most a quarter of what is free, so that programs with many handles or
 // a pool of their own keep the product-by-product path instead of running out. False when
-// there is no room (buf is then empty and no longer counted).
+// there is no room: beyond these limits buf stays what it was, counted, for smaller operators of
+// the same handle (a sweep's next node); where the allocation fails it is empty and not counted.
 bool dense_reserve(attn_ctx* ctx, DevBuf& buf, size_t n, size_t& counted) {
   if (n <= buf.bytes) return true;
   bool ok = ctx->dense_bytes - counted + n <= ctx->total_mem / 16;
@@ -412,7 +413,7 @@ DenseF64* dense_f64(attn_heff* h) {
   const double uses = std::max<double>(h->expect, h->f64_uses > 0 ? 1 + 4.0 * h->f64_uses : 1.0);
   ++h->f64_uses;
   bool use[3];
-  if (!plan_dense(h, uses, use) || stream_capturing(ctx->stream)) return nullptr;
+  if (!plan_dense(h, uses, use) || stream_capturing(ctx->stream) || !h->f64_retry.due()) return nullptr;
   if (!h->dense) h->dense = new DenseF64();
   DenseF64* d = h->dense;
   d->ctx = ctx;
@@ -422,7 +423,11 @@ DenseF64* dense_f64(attn_heff* h) {
     d->at[k] = need;
     if (use[k]) need += pq * pq;
   }
-  if (!dense_reserve(ctx, d->buf, sizeof(double) * need, d->bytes)) return nullptr;
+  if (!dense_reserve(ctx, d->buf, sizeof(double) * need, d->bytes)) {
+    h->f64_retry.failed();
+    return nullptr;
+  }
+  h->f64_retry = DenseRetry();
   PairOps ops;
   ops.n = 0;
   int tiles = 0;
@@ -601,14 +606,25 @@ DenseSplit* dense_split(attn_heff* h) {
     need += ozaki_slice_bytes(parts, pq, kpart[k], 128);
     ne += (size_t)(parts * pq);
   }
-  if (!any || uses * gain < build || stream_capturing(ctx->stream)) return nullptr;
+  if (!any || uses * gain < build || stream_capturing(ctx->stream) || !h->split_retry.due()) return nullptr;
   if (!h->dense_s) h->dense_s = new DenseSplit();
   DenseSplit* d = h->dense_s;
   d->ctx = ctx;
-  if (!dense_reserve(ctx, d->slices, need, d->bytes)) return nullptr;
+  if (!dense_reserve(ctx, d->slices, need, d->bytes)) {
+    h->split_retry.failed();
+    return nullptr;
+  }
   bool hint_done[3] = {false, false, false};
   try {
+    // all memory before any work
     d->exps.reserve(sizeof(int) * ne);
+    size_t most = 0;
+    for (int k = 0; k < 3; ++k) {
+      const long P = h->m[kPairP[k]], Q = h->m[kPairQ[k]];
+      if (use[k]) most = std::max(most, (size_t)(std::min(stage_rows((int)P, (int)Q), P * Q) * P * Q));
+    }
+    ctx->ws[0].reserve(sizeof(double) * most);
+    double* stage = ctx->ws[0].as<double>();
     for (int k = 0; k < 3; ++k) {
       d->use[k] = use[k];
       d->at[k] = at[k];
@@ -622,8 +638,6 @@ DenseSplit* dense_split(attn_heff* h) {
       const double* hq = h->has_hint[q] && !hint_done[q] ? h->hint[q].as<double>() : nullptr;
       hint_done[p] = hint_done[q] = true;
       const long rows = stage_rows(P, Q);
-      ctx->ws[0].reserve(sizeof(double) * (size_t)std::min(rows, PQ) * PQ);
-      double* stage = ctx->ws[0].as<double>();
       for (long r0 = 0; r0 < PQ; r0 += rows) {
         const long r1 = std::min(PQ, r0 + rows);
         // M[(i, j)][(i', j')] = sum_r A_r[i][i'] B_r[j][j'], a batch entry per (i, j): all whole i at once,
@@ -664,8 +678,10 @@ DenseSplit* dense_split(attn_heff* h) {
     d->slices.release();
     ctx->dense_bytes -= d->bytes;
     d->bytes = 0;
+    h->split_retry.failed();
     return nullptr;
   }
+  h->split_retry = DenseRetry();
   for (int s = 0; s < 3; ++s) d->hint[s] = hint_done[s];
   ATTN_CHECK_CUDA(cudaGetLastError());
   d->ready = true;

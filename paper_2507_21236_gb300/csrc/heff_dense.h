@@ -33,6 +33,21 @@ struct DenseSplit {
   ~DenseSplit();
 };
 
+// When to ask again for memory that was refused: at the next application the first three times, then
+// after ever more of them (1, 2, 4 .. 64), since every attempt may allocate and free gigabytes.
+struct DenseRetry {
+  int refused = 0, wait = 0;
+  bool due() {
+    if (wait == 0) return true;
+    --wait;
+    return false;
+  }
+  void failed() {
+    if (refused < 10) ++refused;
+    wait = (1 << refused) / 16;
+  }
+};
+
 // buf of at least n bytes within the context's share of device memory for dense operators;
 // `counted` is what buf has in that count.
 bool dense_reserve(attn_ctx* ctx, DevBuf& buf, size_t n, size_t& counted);
