@@ -166,7 +166,8 @@ ATTN_API attn_status attn_kernel_launches(attn_ctx* ctx, uint64_t* count);
  * stream time (ms, for a phase including any idle gaps between its launches),
  * the number of recorded launches or phases and, for kernels, their algorithmic
  * FLOPs (Sec. 4.4.2 counting: 2 m_l V per operator applied on link l of a tensor
- * of V entries). */
+ * of V entries, also where an FP64 application goes through the sum of a link pair's
+ * products, which takes fewer; making the sums is recorded with its time and no FLOPs). */
 ATTN_API attn_status attn_profile_enable(attn_ctx* ctx, int enable);
 ATTN_API attn_status attn_profile_read(attn_ctx* ctx, int kernel_id, double* total_ms, int* launches, double* flops);
 

@@ -152,6 +152,7 @@ struct GemmF64 {
   long cS = 0;
   // the contraction may run as exact BF16 slice products when attn_config.f64_split is set
   bool split_ok = false;
+  bool counted = true;  // FLOPs of the profile record (false: a preparation, time only)
   // entry of A and of B of batch entry bh (device, Bhi each; null: entry bh); not with split_ok
   const int* aIdx = nullptr;
   const int* bIdx = nullptr;

@@ -301,7 +301,7 @@ void gemm_f64(attn_ctx* ctx, const GemmF64& g0) {
     ATTN_CHECK_CUDA(launch_gemm(ctx->stream, g));
     ctx->launches++;
   }
-  ctx->prof_end(1, fl);
+  ctx->prof_end(1, g0.counted ? fl : 0.0);
   ATTN_CHECK_CUDA(cudaGetLastError());
 }
 

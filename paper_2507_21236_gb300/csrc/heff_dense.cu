@@ -452,11 +452,24 @@ DenseF64* dense_f64(attn_heff* h) {
     tiles += o.tiles_n * ((o.P * o.P + kBT - 1) / kBT);
   }
   for (int s = 0; s < 3; ++s) d->hint[s] = hint_done[s];
+  ctx->prof_begin(1);
   pair_operator_kernel<<<tiles, 256, 0, ctx->stream>>>(ops);
+  ctx->prof_end(1, 0.0);
   ctx->launches++;
   ATTN_CHECK_CUDA(cudaGetLastError());
   d->ready = true;
   return d;
+}
+
+// Algorithmic FLOPs that one application through the sum of kind k stands for: its products one by one
+// (2 m_l V per operator), and with the first such kind the internal operators in the sums.
+static double products_flops(const attn_heff* h, int k, const bool (&use)[3], const bool (&hint)[3]) {
+  double fl = 2.0 * h->npair[k] * (h->m[kPairP[k]] + h->m[kPairQ[k]]) * h->V;
+  for (int q = 0; q < k; ++q)
+    if (use[q]) return fl;
+  for (int s = 0; s < 3; ++s)
+    if (hint[s] && h->has_hint[s]) fl += 2.0 * h->m[s] * h->V;
+  return fl;
 }
 
 // y = (dense kinds) x; every entry of y is written.
@@ -466,8 +479,7 @@ void dense_apply_f64(attn_heff* h, const DenseF64* d, const double* x, double* y
   double fl = 0.0;
   for (int k = 0; k < 3; ++k) {
     g.m[k] = d->use[k] ? d->m(k) : nullptr;
-    const double pq = (double)h->m[kPairP[k]] * h->m[kPairQ[k]];
-    if (d->use[k]) fl += 2.0 * pq * pq * h->m[kPairS[k]];
+    if (d->use[k]) fl += products_flops(h, k, d->use, d->hint);
     g.d[k] = h->m[k];
   }
   g.x = x;
@@ -647,6 +659,7 @@ DenseSplit* dense_split(attn_heff* h) {
           const bool whole = j == 0 && r1 - r >= Q;
           GemmF64 g;
           g.split_ok = true;
+          g.counted = false;
           g.M = P; g.N = Q; g.K = R;
           g.Bhi = whole ? (int)((r1 - r) / Q) : 1;
           g.Blo = whole ? Q : (int)std::min<long>(Q - j, r1 - r);
@@ -713,7 +726,8 @@ void dense_apply_split(attn_heff* h, const DenseSplit* d, const double* x, doubl
     q.nblo = parts.n[k];
     const long pq = (long)h->m[kPairP[k]] * h->m[kPairQ[k]];
     gemm_f64_presliced(ctx, reinterpret_cast<const __nv_bfloat16*>(d->slices.as<uint8_t>() + d->at[k]),
-                       d->exps.as<int>() + d->eat[k], (int)pq, q, ctx->ws[0].as<double>() + off[k]);
+                       d->exps.as<int>() + d->eat[k], (int)pq, q, ctx->ws[0].as<double>() + off[k],
+                       products_flops(h, k, d->use, d->hint));
   }
   dim3 grid((m2 + 31) / 32, (m1 + 31) / 32, m0);
   split_combine_kernel<<<grid, dim3(32, 8), 0, ctx->stream>>>(y, m0, m1, m2, parts);

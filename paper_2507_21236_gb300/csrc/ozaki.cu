@@ -731,7 +731,8 @@ int oz_kparts(int M, int N, long K, int sms) {
   return 64 * at;
 }
 
-void gemm_f64_presliced(attn_ctx* ctx, const __nv_bfloat16* ps, const int* pe, int M, const OzView& q, double* C) {
+void gemm_f64_presliced(attn_ctx* ctx, const __nv_bfloat16* ps, const int* pe, int M, const OzView& q, double* C,
+                        double flops) {
   oz_prepare(ctx);
   const long nkb = q.kpart / 64;
   const int nrtP = (M + 127) / 128, nrtQ = (q.rows + kQRows - 1) / kQRows;
@@ -751,7 +752,7 @@ void gemm_f64_presliced(attn_ctx* ctx, const __nv_bfloat16* ps, const int* pe, i
   prm.C = C; prm.c_rs = 1; prm.c_cs = M; prm.c_bhi = 0; prm.c_blo = (long)M * q.rows;
   prm.alpha_rest = 1.0; prm.alpha_exp = 0; prm.beta = 0.0;
   oz_launch(ctx, maps, prm);
-  ctx->prof_end(3, 2.0 * M * q.rows * (double)q.K * q.G);
+  ctx->prof_end(3, flops);
   ATTN_CHECK_CUDA(cudaGetLastError());
 }
 
@@ -856,7 +857,7 @@ void gemm_f64_ozaki(attn_ctx* ctx, const GemmF64& g0) {
     }
     oz_launch(ctx, maps, prm);
   }
-  ctx->prof_end(3, fl);
+  ctx->prof_end(3, g0.counted ? fl : 0.0);
   ATTN_CHECK_CUDA(cudaGetLastError());
 }
 

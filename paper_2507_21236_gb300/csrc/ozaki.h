@@ -32,8 +32,9 @@ size_t ozaki_slice_bytes(long batches, long rows, long Kpad, int tile_rows);
 
 // C[s][j][i] = sum over K part s of P[i][k] Q[j][k] for an operand P of M rows sliced beforehand
 // (ozaki_slice of a view in K parts, 128-row tiles) and a view Q in the same parts: one dense
-// [Q.rows][M] matrix per part, to be added up.
-void gemm_f64_presliced(attn_ctx* ctx, const __nv_bfloat16* ps, const int* pe, int M, const OzView& q, double* C);
+// [Q.rows][M] matrix per part, to be added up; flops: what the profile records for it.
+void gemm_f64_presliced(attn_ctx* ctx, const __nv_bfloat16* ps, const int* pe, int M, const OzView& q, double* C,
+                        double flops);
 // Part length for an M x N product over K: 4 to 16 K blocks, the fewest on the busiest SM. Short
 // parts also keep the error down: what the scheme drops goes with the product of the row
 // scales, and the largest of 1024 entries exceeds the typical one by less than that of 16384
