@@ -307,7 +307,12 @@ ATTN_API attn_status attn_heff_info(attn_heff* h, int n_pair[3], int* n_triple, 
  * products when the context's f64_split is set), or ATTN_BF16 / ATTN_TF32 operands
  * with FP32 accumulation on the tensor cores, which need every link dimension in
  * {16, 32, ..., 128} (ATTN_EUNSUPPORTED otherwise). Asynchronous on the context
- * stream. */
+ * stream. ATTN_F64 goes product by product or through the sums of the products of each
+ * link pair, which the handle makes and keeps once that pays for the applications made or
+ * announced (a Lanczos depth) and device memory has room: at most a sixteenth of the GPU per
+ * context, beyond 64 MB a quarter of what is free. The two ways agree to rounding, not
+ * bit for bit, so the last bits of equal calls depend on how often the handle was applied
+ * before and, near these limits, on the memory in use. */
 ATTN_API attn_status attn_heff_apply(attn_heff* h, const double* x_dev, double* y_dev, attn_dtype dtype);
 /* Same with host buffers: copies x in, applies, copies y out (synchronous). */
 ATTN_API attn_status attn_heff_apply_host(attn_heff* h, const double* x_host, double* y_host, attn_dtype dtype);
