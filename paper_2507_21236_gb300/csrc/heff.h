@@ -54,6 +54,7 @@ struct attn_heff {
   attn::DenseSplit* dense_s = nullptr;  // the same as BF16 slices (f64_split)
   int f64_uses = 0, split_uses = 0, expect = 1;
   attn::DenseRetry f64_retry, split_retry;
+  bool kept = false;  // its buffers go to a state's next H_eff (allocating them is no cost of this one)
   EigGraph* eg = nullptr; // cached eigensolve graph (use_graphs)
   attn::DevBuf host_x;    // device copy of the tensor of attn_eigsolve_host
   double flops() const;

@@ -370,8 +370,10 @@ DenseSplit::~DenseSplit() {
 // product path (per kind a mode product, a sum over products and its split, and a share of
 // the fill and the internal operators).
 static bool plan_dense(const attn_heff* h, double uses, bool (&use)[3]) {
-  // a handle's first dense operators also cost an allocation
-  double gain = 0.0, build = kLaunch + (h->dense ? 0.0 : kAlloc);
+  // A handle's dense operators also cost an allocation; one that a state keeps for its local steps
+  // counts none, not even the first time: its choice must not depend on what the state did before,
+  // so that a resumed run repeats the original's bits.
+  double gain = 0.0, build = kLaunch + (h->kept ? 0.0 : kAlloc);
   bool any = false;
   for (int k = 0; k < 3; ++k) {
     const double P = h->m[kPairP[k]], Q = h->m[kPairQ[k]], S = h->m[kPairS[k]], R = h->npair[k];

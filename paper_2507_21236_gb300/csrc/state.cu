@@ -448,6 +448,7 @@ attn_heff* attn_state::build_heff(int n) {
   for (int s = 0; s < 3; ++s) E[s] = &get_env(n, s);
   attn_heff* h = spare_heff ? spare_heff : new attn_heff();
   spare_heff = nullptr;
+  h->kept = false;
   h->ctx = ctx;
   for (int s = 0; s < 3; ++s) h->m[s] = dim(n, s);
   h->V = vol(n);
@@ -512,6 +513,7 @@ attn_heff* attn_state::build_heff(int n) {
 
 double attn_state::energy() {
   attn_heff* h = build_heff(centre);
+  h->kept = true;
   const long V = vol(centre);
   lw.wvec.reserve(sizeof(double) * V);
   ctx->scal.reserve(sizeof(double) * 64);
@@ -538,6 +540,7 @@ double attn_state::local_step(int n) {
   ctx->prof_end(4, 0.0);
   ctx->prof_begin(5);
   attn_heff* h = build_heff(n);
+  h->kept = true;
   ctx->prof_end(5, 0.0);
   const long V = vol(n);
   double result = 0.0;
