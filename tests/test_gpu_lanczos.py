@@ -54,3 +54,52 @@ def test_lowest_pair(shape, graph):
             assert abs(abs(u[:, 0] @ v.ravel()) - 1.0) < 1e-10
     attn.attn_heff_destroy(H)
     attn.attn_destroy(ctx)
+
+
+def _bound(V, depth, theta):
+    """Residual after `depth` steps: of the start's part outside the lowest state (0.02 sqrt(V)) each step
+    keeps exp(-2 asinh sqrt(gap / spread)), gap above 4 (6 less what the weak operators shift it by) of a
+    spectrum below 20 wide; and the rounding of the recurrence."""
+    rate = np.exp(-2.0 * np.arcsinh(np.sqrt(4.0 / 20.0)))
+    return 2.0 * 24.0 * 0.02 * np.sqrt(V) * rate ** (depth - 1) + 1e-12 * abs(theta)
+
+
+# 16 CTAs with ceil(V / 16) entries of depth + 1 vectors in 200 KB each: V = 16384 at depth 24 and 19500
+# at depth 20 are the largest that fit, 16275 leaves the last CTA short, the others are beyond it
+@pytest.mark.parametrize("shape,depth", [((16, 32, 32), 24), ((16, 32, 33), 24), ((15, 31, 35), 24), ((25, 26, 30), 20),
+                                         ((25, 26, 31), 20)])
+@pytest.mark.parametrize("graph", [0, 1])
+def test_lowest_pair_at_the_limit_of_the_cluster(shape, depth, graph):
+    attn, ctx = lib_and_ctx({"lanczos_depth": depth, "use_graphs": graph, "lanczos_tol": 0.0})
+    H, start = _heff(attn, ctx, shape, int(sum(shape)), 6.0)
+    for rep in range(2):
+        t = dev(start)
+        theta, iters = attn.attn_eigsolve(H, t)
+        assert iters == depth
+        v = host(t)
+        assert abs(np.linalg.norm(v) - 1.0) < 1e-13
+        assert abs(float((v * attn.attn_heff_apply_host(H, v)).sum()) - theta) <= 1e-12 * abs(theta)
+        assert _residual(attn, H, v, theta) <= _bound(np.prod(shape), depth, theta)
+    attn.attn_heff_destroy(H)
+    attn.attn_destroy(ctx)
+
+
+@pytest.mark.parametrize("shape,depth", [((16, 16, 16), 24), ((32, 32, 32), 24), ((32, 32, 48), 24), ((32, 32, 32), 20)])
+def test_fp32_basis_at_the_limit_of_the_cluster(shape, depth):
+    """TF32 matvecs: 32768 entries are the largest whose FP32 basis fits at depth 24. The Ritz value agrees
+    with the FP64 basis's to the FP32 rounding of each of the basis vectors. (No residual: the operator
+    rounds its input to TF32, so on the Ritz vector it is not the sum of what it gave on the basis.)"""
+    out = {}
+    for basis in (0, 1):
+        attn, ctx = lib_and_ctx({"lanczos_depth": depth, "lanczos_tol": 0.0, "matvec_dtype": 2, "refine_steps": 0,
+                                 "lanczos_basis": basis})
+        H, start = _heff(attn, ctx, shape, int(sum(shape)), 6.0)
+        t = dev(start)
+        theta, _ = attn.attn_eigsolve(H, t)
+        v = host(t)
+        assert abs(np.linalg.norm(v) - 1.0) <= depth * 2.0 ** -23
+        single = depth * 2.0 ** -22 * abs(theta)  # (FP32 sums in the operator itself, in both)
+        out[basis] = theta
+        attn.attn_heff_destroy(H)
+        attn.attn_destroy(ctx)
+    assert abs(out[1] - out[0]) <= single
