@@ -228,7 +228,9 @@ cudaError_t launch_gemm(cudaStream_t stream, const GemmF64& g) {
   return cudaGetLastError();
 }
 
-// Resident CTAs per SM of the tile shape launch_gemm picks for g (queried once per shape).
+// Resident CTAs per SM of the 32- or 64-wide tile that fits g, with which gemm_f64 decides on a split
+// (queried once per shape). An estimate: launch_gemm picks its tile afterwards (tile_of), narrower ones
+// where that evens out the SMs.
 static int resident_ctas(const GemmF64& g) {
   static int occ[4] = {0, 0, 0, 0};
   const int v = (g.M <= 32 ? 2 : 0) + (g.N <= 32 ? 1 : 0);
@@ -262,8 +264,8 @@ void gemm_f64(attn_ctx* ctx, const GemmF64& g0) {
   const long nb = (long)g0.Bhi * g0.Blo;
   const long tiles = (long)((g0.N + bn - 1) / bn) * ((g0.M + bm - 1) / bm) * nb;
   const long slots = (long)std::max(ctx->num_sms, 1) * resident_ctas(g0);
-  // split the G reduction when the output tiles fill less than half a wave: as many
-  // groups as keep the whole grid within one wave of resident CTAs. A reduction over K alone is
+  // split the G reduction when the output tiles (32 or 64 wide) fill less than half a wave: as many
+  // groups as keep a grid of these tiles within one wave of resident CTAs. A reduction over K alone is
   // first cut into equal pieces of at least 32, from K = 256 on (the renormalised internal operator of a link is
   // one 64 x 64 product over K = 4096: 4.0 ms on the one SM that had it, 0.06 ms over all)
   GemmF64 g = g0;

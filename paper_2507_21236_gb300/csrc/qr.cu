@@ -274,7 +274,7 @@ struct QrShared {
   double loc[2][2 * kQrMaxK];  // this CTA's sums (two, so that one cluster barrier suffices)
   double tot[2 * kQrMaxK];     // sums over all rows
   double sum[2 * kQrT];        // partial sums of thread groups
-  double nrm0[kQrMaxK], rprev[kQrMaxK], coef[kQrMaxK];
+  double nrm0[kQrMaxK], rprev[kQrMaxK];
   double rho, inv, sy;  // of the column being completed
   int again, dead;
 };

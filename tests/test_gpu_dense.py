@@ -42,7 +42,7 @@ def _abs(t):
     return np.abs(t) if isinstance(t, np.ndarray) else tuple(np.abs(v) for v in t)
 
 
-# block edges (4 and 8 wide), K steps of 32, single rows, missing kinds, triples, every block size
+# block edges (4 and 8 wide), K steps of 64 and 128, single rows, missing kinds, triples, every block size
 CASES = [((2, 2, 4), (3, 2, 5), 0), ((4, 4, 16), (9, 0, 7), 2), ((16, 16, 16), (12, 12, 14), 0),
          ((5, 7, 9), (11, 30, 8), 3), ((1, 33, 17), (20, 0, 40), 0), ((32, 31, 33), (40, 45, 50), 1),
          ((24, 48, 40), (70, 1, 65), 0), ((64, 72, 80), (90, 100, 80), 0)]

@@ -1,6 +1,6 @@
 """BF16 and TF32 H_eff at links of at most 64 against the products in FP64 (numpy), and against the
-general tensor-core kernel (tc_schedule 1): one to eight slices per unit, slice counts that do not
-divide, missing kinds, three-link products, lists shorter and longer than one run per SM."""
+general tensor-core kernel (tc_schedule 1): four and eight slices per unit, missing kinds, three-link
+products, lists shorter and longer than one run per SM."""
 import numpy as np
 import pytest
 
