@@ -185,7 +185,7 @@ __device__ void mera_solve(const double* G, double* u) {
 // twice (half h of the warp takes every other entry of the environment). An FP64 instruction
 // occupies a warp's scheduler for 64 cycles however many of its lanes work, so a thread
 // doing its matrix products alone costs the same time per multiply-add as 32 of them do here.
-// 16 disentanglers, 20 steps: 4.0 -> 0.41 ms.
+// 12 disentanglers of an 8x8 lattice, 20 steps: 4.0 -> 0.44 ms.
 struct DeShared {
   double u[16], w[2][16], g[16];
   double M[kMaxEnt][16], C[kMaxEnt][16];
